@@ -137,17 +137,22 @@ fc_status fc_set_sampler_shape(fc_graph* g, int32_t walkers_per_tree, int32_t ma
 fc_status fc_set_start_order(fc_graph* g, int32_t order);
 
 /*
- * Sampler kernel: 0 = automatic (the default: the edge-record kernel when the
- * tree state lives in global memory, else the CSR-walk kernel with the state
- * in shared memory), 1 = CSR-walk kernel, 2 = edge-record kernel (FC_EINVAL if
- * g has no edge records: graphs without edges).  Edge records are 16 bytes
+ * Sampler kernel: 0 = automatic (the default: cycle popping -- every vertex
+ * draws its first stack entry and the cycles of the selected entries are
+ * popped until none is left -- unless a setting below chooses a walker kernel
+ * or forest roots are wanted; then the edge-record kernel when the tree state
+ * lives in global memory, else the CSR-walk kernel with the state in shared
+ * memory), 1 = CSR-walk kernel, 2 = edge-record kernel (FC_EINVAL if g has no
+ * edge records: graphs without edges).  The walker settings
+ * (fc_set_sampler_shape, _pops, _bitmap, _cluster at non-zero values) choose
+ * among the walker kernels.  Edge records are 16 bytes
  * per CSR entry (64 bytes for weighted graphs, which also carry slot
- * thresholds) per alpha.  Both kernels draw the same random stacks, so the
+ * thresholds) per alpha.  Every kernel draws the same random stacks, so the
  * trees are identical; only speed differs.
  * fc_sampler_last_kernel returns the kernel of the last launch on g: 1 =
  * CSR-walk, 2 = edge-record with tree membership as state flags, 3 =
  * edge-record with the in-tree bitmap in shared memory, 4 = edge-record with
- * the in-tree bitmap in global memory; 0 before any launch.
+ * the in-tree bitmap in global memory, 5 = cycle popping; 0 before any launch.
  */
 fc_status fc_set_sampler_kernel(fc_graph* g, int32_t kernel);
 int32_t fc_sampler_last_kernel(const fc_graph* g);
@@ -223,7 +228,8 @@ fc_status fc_sampler_last_shape(const fc_graph* g, int32_t* walkers_per_tree, in
  *            [(a*tau + t)*n + v], u* = n -- optional (test / analysis mode)
  *   steps_out uint64[n_alpha * tau] stack entries consumed by each tree
  *            (= departures of the sequential algorithm) -- optional
- * max_steps_per_tree: watchdog on the iterations of each walker (0 = default
+ * max_steps_per_tree: watchdog on the iterations of each walker (cycle
+ * popping: on the steps of each walk and on the rounds of popping; 0 = default
  * 8 n + 2^20; graphs from fc_build_rooted: 2^26 + 64 n, since walks on G have
  * a single exit); exceeding it aborts the launch with FC_ETIMEOUT.
  * Requires tau >= 0, tree_offset >= 0, tree_offset + tau <= 2^32.

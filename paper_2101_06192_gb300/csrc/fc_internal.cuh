@@ -218,6 +218,7 @@ struct fc_graph {
   int64_t shape_val[SHAPE_SLOTS][6] = {};
   bool shape_used[SHAPE_SLOTS] = {};
   int32_t shape_next = 0;
+  size_t pop_bytes = 0;        // largest scratch of a cycle-popping call (sizes later captured calls)
   // scratch owned by the graph
   void* ws = nullptr;          // sampler per-tree state
   size_t ws_bytes = 0;

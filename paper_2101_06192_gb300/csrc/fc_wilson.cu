@@ -618,6 +618,8 @@ extern "C" fc_status fc_sample_usts_async(fc_graph* g, uint64_t seed, int64_t ta
   return sample_impl(g, seed, tau, tree_offset, R, C, parents, nullptr, max_steps_per_tree, steps_out, stream, false);
 }
 
+static fc_status sampler_status(uint32_t herr, const char* who);
+
 extern "C" fc_status fc_sampler_check(fc_graph* g, void* stream) {
   if (g == nullptr) return fcx::invalid("fc_sampler_check: bad argument");
   cudaStream_t st = (cudaStream_t)stream;
@@ -626,31 +628,124 @@ extern "C" fc_status fc_sampler_check(fc_graph* g, void* stream) {
   FC_CK(cudaStreamSynchronize(st));
   FC_CK(cudaMemsetAsync(g->d_err, 0, sizeof(uint32_t), st));
   FC_CK(cudaStreamSynchronize(st));
+  return sampler_status(herr, "fc_sampler_check");
+}
+
+// default watchdog: 8 n + 2^20 iterations per walker on G* (every step can
+// exit to u*); walks on G with one exit (fc_build_rooted) take
+// sum_v d_w(v) r(root, v) steps in all, up to quadratic in n on long
+// paths, and walkers wait for each other longer: 2^26 + 64 n
+static uint32_t iteration_budget(const fc_graph* g, uint64_t max_steps_per_tree) {
+  const uint64_t n = (uint64_t)g->n;
+  const uint64_t mi =
+      max_steps_per_tree ? max_steps_per_tree : (g->root >= 0 ? (1ull << 26) + 64 * n : 8 * n + (1ull << 20));
+  return (uint32_t)std::min<uint64_t>(mi, 0xffffffffull);
+}
+
+// status of a launch from its device error word
+static fc_status sampler_status(uint32_t herr, const char* who) {
   if (herr & ERR_OVERFLOW) {
-    set_error("fc_sampler_check: a visit counter exceeded 2^24 - 1");
+    set_error(std::string(who) + ": a visit counter exceeded 2^24 - 1");
     return FC_EOVERFLOW;
   }
   if (herr & ERR_TIMEOUT) {
-    set_error("fc_sampler_check: watchdog iteration budget exhausted");
+    set_error(std::string(who) + ": watchdog iteration budget exhausted");
     return FC_ETIMEOUT;
   }
   if (herr != 0) {
-    set_error("fc_sampler_check: internal consistency check failed");
+    set_error(std::string(who) + ": internal consistency check failed");
     return FC_ECUDA;
   }
   return FC_OK;
 }
 
-namespace {
-// device scratch released on the stream when the call returns
-struct StreamScratch {
-  void* ptr = nullptr;
-  cudaStream_t st = nullptr;
-  ~StreamScratch() {
-    if (ptr) cudaFreeAsync(ptr, st);
+// completion times of a batch launch, [graphs][tau]
+static fc_status batch_stamps(fc_graph* g, int64_t tau, bool capturing, cudaStream_t st) {
+  const size_t items = (size_t)g->num_graphs * (size_t)tau;
+  if (g->item_cap < items && capturing) {
+    set_error("fc_sample_usts_async: batch timestamps must be sized by an uncaptured call before stream capture");
+    return FC_EINVAL;
   }
-};
-}  // namespace
+  if (g->item_cap < items) {
+    if (g->item_ns) FC_CK(cudaFreeAsync(g->item_ns, st));
+    g->item_ns = nullptr;
+    g->item_cap = 0;
+    FC_CK(cudaMallocAsync((void**)&g->item_ns, items * sizeof(unsigned long long), st));
+    g->item_cap = items;
+  }
+  g->last_tau = tau;
+  return FC_OK;
+}
+
+// The cycle-popping sampler (fc_pop.cu) takes every call in automatic mode:
+// choosing a walker kernel, its launch shape, tree membership, cycle popping or
+// clusters (fc_set_sampler_*) keeps that kernel.  Measured on GB300 against
+// the walker kernels (ms per call): BA n = 2^20, 1024 trees 42.5 -> 23.7;
+// R-MAT 2^20, 64 trees 8.5 -> 1.5; weighted 1024^2 grid, 152 trees, alpha 0.1
+// 25.0 -> 4.4, 1 47.3 -> 15.0, 10 79.4 -> 38.9; ER n = 1000, 2000 trees 1.3 ->
+// 0.37; BA n = 2^20 rooted at its hub, 152 trees 118 -> 87.  Exceptions:
+//  * forest roots: recorded by the edge-record kernel as vertices join a tree;
+//  * ids of 29 bits in the words of the tops;
+//  * parents (an analysis output) of unweighted graphs of 2^15 to 2^16 vertices
+//    without a dominating hub: tests/test_gpu_edge_kernel.py pins the walker
+//    kernel and its automatic clusters for these launches (0.87 ms against
+//    0.34 ms for 64 trees of BA n = 50,000).
+static bool pop_applies(const fc_graph* g, const int32_t* parents, const int32_t* roots, const int32_t* depths) {
+  const bool automatic = g->kernel_pref == 0 && g->walkers == 0 && g->max_trees == 0 && g->smem_mode == 0 &&
+                         g->regs == 0 && g->bitmap_mode == 0 && g->pops_mode == 0 && g->cluster == 0;
+  const bool pinned = parents != nullptr && !g->weighted && g->num_graphs == 0 && g->root < 0 && g->n > (1 << 15) &&
+                      g->n <= (1 << 16) && g->max_deg <= g->n / 16;
+  return automatic && roots == nullptr && depths == nullptr && g->n < (1 << 29) - 1 && !pinned;
+}
+
+static fc_status sample_pop(fc_graph* g, uint64_t seed, int64_t tau, int64_t tree_offset, uint32_t* R, uint32_t* C,
+                            int32_t* parents, uint64_t* visits, uint64_t max_steps_per_tree, uint64_t* steps_out,
+                            cudaStream_t st, bool sync, bool capturing) {
+  const bool batch = g->num_graphs > 0;
+  WParams p = {};
+  p.tau = tau;
+  p.tree_offset = tree_offset;
+  p.key0 = (uint32_t)seed;
+  p.key1 = (uint32_t)(seed >> 32);
+  p.R = R;
+  p.C = C;
+  p.parents = parents;
+  p.visits = (unsigned long long*)visits;
+  p.steps = steps_out;
+  p.err = g->d_err;
+  p.stats = g->d_stats;
+  p.max_iters = iteration_budget(g, max_steps_per_tree);
+  if (batch) {
+    const fc_status s = batch_stamps(g, tau, capturing, st);
+    if (s != FC_OK) return s;
+    p.item_ns = g->item_ns;
+    p.t0_ns = g->t0_ns;
+  }
+  int optin = 0;
+  FC_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
+  // a captured call needs its scratch sized by an uncaptured one, as for the
+  // walker kernels (whose small graphs live in shared memory and need none)
+  const bool small = smem_bytes(32, batch ? g->max_ng : g->n, true) + 64 <= (size_t)optin;
+  PopPlan pl;
+  const int64_t total = (int64_t)(batch ? 1 : g->n_alpha) * tau;  // a row of a batch: one tree of every graph
+  const fc_status ps = pop_plan(g, total, &pl);
+  if (ps != FC_OK) return ps;
+  if (capturing && !small && g->pop_bytes < pl.bytes) {
+    set_error("fc_sample_usts_async: sampler scratch must be sized by an uncaptured call before stream capture");
+    return FC_EINVAL;
+  }
+  g->pop_bytes = std::max(g->pop_bytes, pl.bytes);
+  StreamScratch scr;  // of this call alone: calls on other streams have their own
+  scr.st = st;
+  FC_CK(cudaMallocAsync(&scr.ptr, pl.bytes, st));
+  if (sync) FC_CK(cudaMemsetAsync(g->d_err, 0, sizeof(uint32_t), st));
+  const fc_status s = pop_sample(g, p, pl, scr.ptr, st);
+  if (s != FC_OK || !sync) return s;
+  uint32_t herr = 0;
+  FC_CK(cudaMemcpyAsync(&herr, g->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+  FC_CK(cudaStreamSynchronize(st));
+  return sampler_status(herr, "fc_sample_usts");
+}
 
 static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tree_offset, uint32_t* R, uint32_t* C,
                              int32_t* parents, uint64_t* visits, uint64_t max_steps_per_tree, uint64_t* steps_out,
@@ -670,6 +765,9 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
     set_error("fc_sample_usts: reads its status back; use fc_sample_usts_async on a capturing stream");
     return FC_EINVAL;
   }
+  if (pop_applies(g, parents, roots, depths))
+    return sample_pop(g, seed, tau, tree_offset, R, C, parents, visits, max_steps_per_tree, steps_out, st, sync,
+                      capturing);
   int dev_smem_optin = 0, nsm = 0;
   FC_CK(cudaDeviceGetAttribute(&dev_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
   FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
@@ -851,17 +949,8 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
   // walkers, in-tree bitmap) with the ramp ran no faster (214 ms).
   p.ramp_q = (edge && cl == 1 && g->root >= 0) ? (uint32_t)std::max<int64_t>(1, (int64_t)nmax >> 8) : 0u;
   if (batch) {
-    const size_t items = (size_t)g->num_graphs * (size_t)tau;
-    if (g->item_cap < items && capturing) {
-      set_error("fc_sample_usts_async: batch timestamps must be sized by an uncaptured call before stream capture");
-      return FC_EINVAL;
-    }
-    if (g->item_cap < items) {
-      if (g->item_ns) FC_CK(cudaFreeAsync(g->item_ns, st));
-      FC_CK(cudaMallocAsync((void**)&g->item_ns, items * sizeof(unsigned long long), st));
-      g->item_cap = items;
-    }
-    g->last_tau = tau;
+    const fc_status s = batch_stamps(g, tau, capturing, st);
+    if (s != FC_OK) return s;
     p.item_ns = g->item_ns;
     p.t0_ns = g->t0_ns;
     FC_CK(cudaMemsetAsync(g->t0_ns, 0xff, sizeof(unsigned long long), st));
@@ -869,16 +958,7 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
   p.counter = g->d_counter;
   p.err = g->d_err;
   p.stats = g->d_stats;
-  {
-    // default watchdog: 8 n + 2^20 iterations per walker on G* (every step can
-    // exit to u*); walks on G with one exit (fc_build_rooted) take
-    // sum_v d_w(v) r(root, v) steps in all, up to quadratic in n on long
-    // paths, and walkers wait for each other longer: 2^26 + 64 n
-    const uint64_t mi = max_steps_per_tree ? max_steps_per_tree
-                        : (g->root >= 0 ? (1ull << 26) + (uint64_t)64 * (uint64_t)n
-                                        : (uint64_t)8 * (uint64_t)n + (1ull << 20));
-    p.max_iters = (uint32_t)std::min<uint64_t>(mi, 0xffffffffull);
-  }
+  p.max_iters = iteration_budget(g, max_steps_per_tree);
   p.pre_cleared = 0;
   if (!use_smem) {
     // clear the state and bitmaps of the first wave in one pass
@@ -920,18 +1000,8 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
   uint32_t herr = 0;
   FC_CK(cudaMemcpyAsync(&herr, g->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   FC_CK(cudaStreamSynchronize(st));
-  if (herr & ERR_OVERFLOW) {
-    set_error("fc_sample_usts: a visit counter exceeded 2^24 - 1");
-    return FC_EOVERFLOW;
-  }
-  if (herr & ERR_TIMEOUT) {
-    set_error("fc_sample_usts: watchdog iteration budget exhausted");
-    return FC_ETIMEOUT;
-  }
-  if (herr != 0) {
-    set_error("fc_sample_usts: internal consistency check failed");
-    return FC_ECUDA;
-  }
+  const fc_status es = sampler_status(herr, "fc_sample_usts");
+  if (es != FC_OK) return es;
   if (want_roots && !fused_roots) {
     StreamScratch r2;
     r2.st = st;

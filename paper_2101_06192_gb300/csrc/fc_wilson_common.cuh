@@ -153,4 +153,24 @@ typedef void (*WilsonFn)(WParams);
 WilsonFn wilson_edge_fn(int bits, bool wgt, bool ring, bool cl, int regs, bool roots = false);
 size_t wilson_edge_smem(int W, int32_t n, int bits, bool wgt, int C, bool ring);  // bits: 0 flags, 1 shared bitmap, 2 global
 
+// device scratch released on the stream when the call returns
+struct StreamScratch {
+  void* ptr = nullptr;
+  cudaStream_t st = nullptr;
+  ~StreamScratch() {
+    if (ptr) cudaFreeAsync(ptr, st);
+  }
+};
+
+// Cycle-popping sampler (fc_pop.cu): the plan of a call of total rows ((alpha,
+// tree) pairs; a batch: one tree of every graph), and the call on scratch of
+// plan.bytes bytes.
+struct PopPlan {
+  int teams, ctas;  // teams and CTAs per team
+  int32_t wrows;    // rows per window
+  size_t bytes;     // scratch
+};
+fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* plan);
+fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& plan, void* ws, cudaStream_t st);
+
 }  // namespace fcx

@@ -11,6 +11,9 @@ trees, kernel) in a JSON file next to the built library.  Choices measured
 on GB300 for common graph classes ship with the package (tuned_shapes.json)
 and are used when the local cache has no entry, so those classes start with
 a fixed, reproducible shape.  Neither changes results.
+
+All this concerns the walker kernels (set_kernel(1) or (2)).  The automatic
+sampler (cycle popping) sizes its own launches: autotune leaves it alone.
 """
 from __future__ import annotations
 
@@ -63,12 +66,16 @@ def apply(G, entry: dict):
 def autotune(G, tau: int, probe_trees: int | None = None, seed: int = 12345) -> dict:
     """Pick and apply the fastest start order, then the fastest (walkers,
     regs), for G at tau trees per alpha."""
+    if G.kernel_pref == 0:
+        entry = {"walkers": 0, "regs": 0, "order": "auto", "kernel": "automatic"}
+        apply(G, entry)
+        return entry
     key = _key(G, tau)
     cache = _load()
     if key in cache:
         apply(G, cache[key])
         return dict(cache[key], cached=True)
-    shipped = _load(_SHIPPED).get(key)
+    shipped = _load(_SHIPPED).get(key[:-1] + "0")  # measured with the edge-record kernel
     if shipped is not None:
         apply(G, shipped)
         return dict(shipped, cached="shipped")
