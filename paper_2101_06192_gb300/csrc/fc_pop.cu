@@ -32,9 +32,17 @@
 // that selects u* is final (it is never on a cycle), so R, C and the
 // departures are counted where entries are drawn.
 //
-// The CTAs of one cooperative launch form teams of one CTA per SM with their
-// own barriers; each team takes its own windows, so while one team waits for
-// its longest walk (a chain of dependent loads) the others fill the SMs.
+// The CTAs of one cooperative launch form teams with their own barriers; each
+// team takes its own windows, so while one team waits for its longest walk (a
+// chain of dependent loads) the others fill the SMs.
+//
+// What bounds it (GB300, BA n = 2^20, mean degree 16; 160 trees, phases timed as
+// launches of their own): drawing 3.7 us per tree, issue (131 warp instructions
+// per 32 vertices, most of them Philox); first walks 6.0 us, latency of 0.7 n
+// dependent 4-byte gathers (110 G/s of the 290 G/s that independent gathers
+// reach); redraws 3.9 us, DRAM (290 bytes per listed vertex at 4.8 TB/s: word,
+// row info and target lie in different sectors); later rounds 5 us.  The walker
+// kernels took 41 us per tree, 570 warp instructions per iteration.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -48,10 +56,13 @@ namespace {
 constexpr uint32_t PW_RED = 1u << 29;
 constexpr uint32_t PW_ACT = 1u << 30;  // shifted by the round's parity
 constexpr uint32_t PW_ID = PW_RED - 1u;
+constexpr uint32_t PW_NONE = 0xffffffffu;
 constexpr int PK_T = 256;      // threads per CTA
 constexpr int PK_W = PK_T / 32;
 constexpr int PK_CHUNK = 256;  // vertices of one row looked at by a warp at a time
-constexpr int PK_EMIT = 128;   // listed vertices buffered by a warp
+constexpr int PK_RING = 512;   // candidates waiting per warp (a power of two, over PK_CHUNK + 32)
+constexpr int PK_OWN = 64;     // finders noted by a warp
+constexpr int PK_STEPS = 4;    // walk steps between two looks for idle lanes
 
 struct PopParams {
   int32_t n;
@@ -65,6 +76,7 @@ struct PopParams {
   int32_t wrows;          // rows per window
   int32_t teams, ctas;    // teams, CTAs per team
   uint32_t ld;            // words per row (a multiple of 4)
+  uint32_t ld_mul, ld_shift;  // division by ld (row_of_item)
   uint32_t* F;            // [teams][wrows][ld] tops
   uint32_t* K;            // [teams][wrows][ld] entries popped (RED vertices)
   uint32_t* L;            // [teams][2][wrows * ld] listed vertices (row * ld + v)
@@ -138,6 +150,25 @@ __device__ __forceinline__ void row_of(const PopParams& p, int64_t g, int32_t* a
   }
 }
 
+// row of a listed vertex (item row * ld + v): a multiply and a shift instead
+// of a division (exact for items below 2^32: floor(i / d) by the round-up
+// method with a 33-bit multiplier folded into an add)
+__device__ __forceinline__ uint32_t row_of_item(const PopParams& p, uint32_t it) {
+  const uint32_t h = __umulhi(it, p.ld_mul);
+  return (((it - h) >> 1) + h) >> p.ld_shift;
+}
+
+// first slot j of a row of d entries with u < b[j] (b[d - 1] = 2^53)
+__device__ __forceinline__ uint32_t slot_search(const uint64_t* b, uint32_t d, uint64_t u) {
+  uint32_t lo = 0, hi = d - 1u;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (u < __ldg(b + mid)) hi = mid;
+    else lo = mid + 1u;
+  }
+  return lo;
+}
+
 // draw: entry 0 of every vertex in rows [g0, g0 + rows); a thread per vertex,
 // the rows in a loop (row info, and a short row's thresholds, in registers;
 // the targets of the row stay in L1).
@@ -195,13 +226,7 @@ __device__ void pop_draw(const PopParams& p, uint32_t* F, int64_t g0, int32_t ro
 #pragma unroll
             for (int j = 0; j < 7; ++j) slot += u >= bv[j] ? 1u : 0u;
           } else {
-            uint32_t lo = 0, hi = ri.y - 1u;
-            while (lo < hi) {
-              const uint32_t mid = (lo + hi) >> 1;
-              if (u < __ldg(b + mid)) hi = mid;
-              else lo = mid + 1u;
-            }
-            slot = lo;
+            slot = slot_search(b, ri.y, u);
           }
           w = (uint32_t)__ldg(col + slot);
         }
@@ -224,17 +249,18 @@ __device__ void pop_draw(const PopParams& p, uint32_t* F, int64_t g0, int32_t ro
 
 // redraw: the next stack entry of every listed vertex; the last round's ACT
 // flags are cleared (a vertex in both lists ends with the new word either way)
+template <bool WGT>
 __device__ void pop_redraw(const PopParams& p, uint32_t* F, uint32_t* K, const uint32_t* list, uint32_t cnt,
                            const uint32_t* old, uint32_t oldcnt, int par, int64_t g0, int cta) {
   const uint32_t stride = (uint32_t)p.ctas * PK_T;
   WParams sp;
-  sp.B = p.B;
+  sp.B = WGT ? p.B : nullptr;
   sp.nnz = p.nnz;
   for (uint32_t i = (uint32_t)cta * PK_T + threadIdx.x; i < oldcnt; i += stride)
     atomicAnd(F + __ldcg(old + i), ~(PW_ACT << (par ^ 1)));
   for (uint32_t i = (uint32_t)cta * PK_T + threadIdx.x; i < cnt; i += stride) {
     const uint32_t it = __ldcg(list + i);
-    const uint32_t r = it / p.ld, v = it - r * p.ld;
+    const uint32_t r = row_of_item(p, it), v = it - r * p.ld;
     int32_t a;
     int64_t t;
     row_of(p, g0 + r, &a, &t);
@@ -255,166 +281,204 @@ __device__ void pop_redraw(const PopParams& p, uint32_t* F, uint32_t* K, const u
   }
 }
 
+// The vertices of the cycles whose finders are listed in own[0, cnt), a lane
+// per cycle: round once for the lengths, once more to append the vertices (the
+// walk that found the cycle left its tops in L1).
+__device__ uint32_t pop_list_cycles(const PopParams& p, const uint32_t* F, const uint32_t* own, int cnt, uint32_t* out,
+                                    uint32_t* outcnt, int64_t g0) {
+  const int lane = threadIdx.x & 31;
+  uint32_t rb = 0, v = 0, len = 0, row = 0;
+  if (lane < cnt) {
+    const uint32_t it = own[lane];
+    row = row_of_item(p, it);
+    rb = row * p.ld;
+    v = it - rb;
+    uint32_t x = v;
+    do {
+      x = ld_top(F + (rb + x)) & PW_ID;
+      ++len;
+    } while (x != v);
+  }
+  __syncwarp();
+  uint32_t s = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(FULL, s, o);
+    if (lane >= o) s += y;
+  }
+  uint32_t b = 0;
+  if (lane == 31) b = atomicAdd(outcnt, s);
+  b = __shfl_sync(FULL, b, 31);
+  if (len) {
+    uint32_t* o = out + (b + s - len);
+    uint32_t x = v;
+    do {
+      *o++ = rb + x;
+      x = ld_top(F + (rb + x)) & PW_ID;
+    } while (x != v);
+    if (p.steps != nullptr) {
+      int32_t a;
+      int64_t t;
+      row_of(p, g0 + row, &a, &t);
+      atomicAdd(p.steps + (p.num_graphs > 0 ? (size_t)p.gid[v] : (size_t)a) * p.tau + (size_t)t,
+                (unsigned long long)len);
+    }
+  }
+  __syncwarp();
+  return len;
+}
+
 // walk: FIRST: every vertex of the window, else the listed ones (cnt of them,
 // ACT flag of parity par).  Vertices of the cycles found are appended to out.
 // Returns this thread's count of them.
+//
+// A warp's lanes walk independently and are bound by the latency of the
+// dependent loads, so every lane is kept on a walk: candidates wait in a ring
+// in shared memory, and the words of the next unit (PK_CHUNK vertices of a
+// row, or 32 listed vertices) are loaded while the lanes walk.
 template <bool FIRST>
-__device__ uint32_t pop_walk(const PopParams& p, const uint32_t* F, const uint32_t* list, uint32_t cnt,
-                             int par, uint32_t* out, uint32_t* outcnt, int64_t g0, int32_t rows, int cta, uint2* q,
-                             uint32_t* em) {
+__device__ uint32_t pop_walk(const PopParams& p, const uint32_t* F, const uint32_t* list, uint32_t cnt, int par,
+                             uint32_t* out, uint32_t* outcnt, int64_t g0, int32_t rows, int cta, uint2* q,
+                             uint32_t* own) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const uint32_t n = (uint32_t)p.n, ld = p.ld;
   const uint32_t act = PW_ACT << par;
   const uint32_t cpr = (n + PK_CHUNK - 1) / PK_CHUNK;  // chunks per row
-  const uint64_t units = FIRST ? (uint64_t)cpr * (uint32_t)rows : ((uint64_t)cnt + 31) / 32;
-  const uint64_t nw = (uint64_t)p.ctas * PK_W;
-  uint64_t unit = (uint64_t)(threadIdx.x >> 5) * p.ctas + cta;
-  int qh = 0, qn = 0, ne = 0;  // warp-uniform: queue [qh, qn), buffered vertices
-  uint32_t qb = 0;             // FIRST: row base of the queue
-  bool walk = false, emit = false;
-  uint32_t rb = 0, v = 0, x = 0, tort = 0, lam = 0, pw = 0, iters = 0, clen = 0, pops = 0;
+  const uint32_t units = FIRST ? cpr * (uint32_t)rows : (cnt + 31u) / 32u;
+  const uint32_t nw = (uint32_t)p.ctas * PK_W;
+  uint32_t unit = (threadIdx.x >> 5) * (uint32_t)p.ctas + (uint32_t)cta;  // the unit whose words are in flight
+  uint32_t qh = 0, qn = 0;  // warp-uniform: ring [qh, qn) of candidates {item, selected vertex}
+  int no = 0;               // finders noted
+  bool walk = false;
+  uint32_t rb = 0, v = 0, x = 0, tort = 0, iters = 0, pops = 0;
+
+  // FIRST: words of the unit in flight and its place; else its items and
+  // words, and the items of the unit after it
+  uint4 w4[2];
+  uint32_t ub = 0, v0 = 0, it1 = PW_NONE, w1 = 0, it2 = PW_NONE;
+  auto load_chunk = [&]() {
+    if (unit < units) {
+      const uint32_t row = unit / cpr;
+      ub = row * ld;
+      v0 = (unit - row * cpr) * PK_CHUNK + lane * 4;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        w4[i] = v0 + i * 128 < n ? __ldcg(reinterpret_cast<const uint4*>(F + ub + v0 + i * 128)) : make_uint4(n, n, n, n);
+    }
+  };
+  auto load_item = [&](uint32_t u) {
+    const uint32_t i = u * 32u + lane;
+    return u < units && i < cnt ? __ldcg(list + i) : PW_NONE;
+  };
+  if (FIRST) {
+    load_chunk();
+  } else {
+    it1 = load_item(unit);
+    it2 = unit + nw < units ? load_item(unit + nw) : PW_NONE;
+    if (it1 != PW_NONE) w1 = ld_top(F + it1);
+  }
   for (;;) {
-    // ---- idle lanes take the next vertices ----
-    unsigned idle = __ballot_sync(FULL, !walk);
-    if (idle) {
-      while (qh == qn && unit < units) {
-        qh = qn = 0;
-        if (FIRST) {
-          const uint32_t row = (uint32_t)(unit / cpr);
-          const uint32_t v0 = (uint32_t)(unit - (uint64_t)row * cpr) * PK_CHUNK;
-          qb = row * ld;
-          const uint32_t* src = F + qb;
-          uint4 w4[2];
+    // ---- the arrived unit's candidates, while the ring runs low ----
+    while (qn - qh < 32u && unit < units) {
+      if (FIRST) {
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const uint32_t vv = v0 + i * 128 + lane * 4;
-            w4[i] = vv < n ? __ldcg(reinterpret_cast<const uint4*>(src + vv)) : make_uint4(n, n, n, n);
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const uint32_t vv = v0 + (i >> 2) * 128 + lane * 4 + (i & 3);
-            const uint4 ww = w4[i >> 2];
-            const uint32_t w = (i & 3) == 0 ? ww.x : (i & 3) == 1 ? ww.y : (i & 3) == 2 ? ww.z : ww.w;
-            const bool cand = vv < n && w != n && w > vv;  // a walk that does not stop at once
-            const unsigned m = __ballot_sync(FULL, cand);
-            if (cand) q[qn + __popc(m & lt)] = make_uint2(vv, w);
-            qn += __popc(m);
-          }
-        } else {
-          const uint32_t i = (uint32_t)unit * 32u + lane;
-          uint32_t it = 0, w = n;
-          if (i < cnt) {
-            it = __ldcg(list + i);
-            w = ld_top(F + it) & PW_ID;
-          }
-          const unsigned m = __ballot_sync(FULL, w != n);
-          if (w != n) q[__popc(m & lt)] = make_uint2(it, w);
-          qn = __popc(m);
+        for (int i = 0; i < 8; ++i) {
+          const uint32_t vv = v0 + (i >> 2) * 128 + (i & 3);
+          const uint4 ww = w4[i >> 2];
+          const uint32_t w = (i & 3) == 0 ? ww.x : (i & 3) == 1 ? ww.y : (i & 3) == 2 ? ww.z : ww.w;
+          const bool cand = vv < n && w != n && w > vv;  // a walk that does not stop at once
+          const unsigned m = __ballot_sync(FULL, cand);
+          if (cand) q[(qn + __popc(m & lt)) & (PK_RING - 1)] = make_uint2(ub + vv, w);
+          qn += __popc(m);
         }
         unit += nw;
-        __syncwarp();
+        load_chunk();
+      } else {
+        const uint32_t w = w1 & PW_ID;
+        const bool cand = it1 != PW_NONE && w != n;
+        const unsigned m = __ballot_sync(FULL, cand);
+        if (cand) q[(qn + __popc(m & lt)) & (PK_RING - 1)] = make_uint2(it1, w);
+        qn += __popc(m);
+        unit += nw;
+        it1 = it2;
+        if (it1 != PW_NONE) w1 = ld_top(F + it1);
+        it2 = unit + nw < units ? load_item(unit + nw) : PW_NONE;
       }
-      const int r = __popc(idle & lt);
+      __syncwarp();
+    }
+    // ---- idle lanes take candidates ----
+    const unsigned idle = __ballot_sync(FULL, !walk);
+    if (idle) {
+      const uint32_t r = (uint32_t)__popc(idle & lt);
       if (!walk && r < qn - qh) {
-        const uint2 cw = q[qh + r];
-        if (FIRST) {
-          rb = qb;
-          v = cw.x;
-        } else {
-          rb = cw.x / ld * ld;
-          v = cw.x - rb;
-        }
+        const uint2 cw = q[(qh + r) & (PK_RING - 1)];
+        rb = row_of_item(p, cw.x) * ld;
+        v = cw.x - rb;
         x = tort = cw.y;
-        lam = pw = 2;
         iters = 0;
         walk = true;
       }
       __syncwarp();
-      qh = min(qn, qh + __popc(idle));
-      if (!__any_sync(FULL, walk)) break;
-    }
-    // ---- steps: until a lane is idle and another vertex may be had ----
-#pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      bool put = false;
-      uint32_t pv = 0;
-      if (walk) {
-        const uint32_t w = ld_top(F + rb + x);
-        const uint32_t y = w & PW_ID;
-        if (emit) {
-          put = true;
-          pv = rb + x;
-          ++clen;
-          if (y == v) {  // the cycle is listed
-            emit = walk = false;
-            pops += clen;
-            if (p.steps != nullptr) {
-              int32_t a;
-              int64_t t;
-              row_of(p, g0 + rb / ld, &a, &t);
-              atomicAdd(p.steps + (p.num_graphs > 0 ? (size_t)p.gid[v] : (size_t)a) * p.tau + (size_t)t,
-                        (unsigned long long)clen);
-            }
-          }
-          x = y;
-        } else if (!FIRST && (w & act) && x < v) {
-          walk = false;
-        } else if (y == n || (FIRST && y < v)) {
-          walk = false;
-        } else if (y == v) {  // v's cycle: go round once more and list it
-          emit = true;
-          clen = 1;
-          put = true;
-          pv = rb + v;
-          x = ld_top(F + rb + v) & PW_ID;
-        } else if (y == tort) {
-          walk = false;
-        } else {
-          x = y;
-          if (--lam == 0u) {
-            tort = y;
-            pw <<= 1;
-            lam = pw;
-          }
-        }
-        if (++iters > p.max_iters) {
-          atomicOr(p.err, ERR_TIMEOUT);
-          walk = emit = false;
-        }
+      qh += min(qn - qh, (uint32_t)__popc(idle));
+      if (!__any_sync(FULL, walk)) {
+        if (unit < units) continue;
+        break;
       }
-      const unsigned m = __ballot_sync(FULL, put);
-      if (m) {
-        if (ne + __popc(m) > PK_EMIT) {
-          uint32_t b = 0;
-          if (lane == 0) b = atomicAdd(outcnt, (uint32_t)ne);
-          b = __shfl_sync(FULL, b, 0);
-          for (int i = lane; i < ne; i += 32) out[b + i] = em[i];
-          ne = 0;
-          __syncwarp();
-        }
-        if (put) em[ne + __popc(m & lt)] = pv;
-        ne += __popc(m);
+    }
+    // ---- a few steps ----
+    bool found = false;
+#pragma unroll
+    for (int s = 0; s < PK_STEPS; ++s) {
+      if (walk) {
+        const uint32_t w = ld_top(F + (rb + x));
+        const uint32_t y = w & PW_ID;
+        bool stop = y == n || y == tort;
+        if (FIRST) stop |= y < v;
+        else stop |= (w & act) != 0u && x < v;
+        found = !stop && y == v;
+        walk = !stop && y != v;
+        x = y;
+        ++iters;
+        if ((iters & (iters - 1u)) == 0u) tort = y;  // Brent: a new reference at every power of two
+      }
+    }
+    if (iters > p.max_iters) {
+      atomicOr(p.err, ERR_TIMEOUT);
+      walk = false;
+    }
+    const unsigned m = __ballot_sync(FULL, found);
+    if (m) {
+      if (found) own[no + __popc(m & lt)] = rb + v;
+      no += __popc(m);
+      __syncwarp();
+      if (no >= 32) {
+        pops += pop_list_cycles(p, F, own + (no - 32), 32, out, outcnt, g0);
+        no -= 32;
         __syncwarp();
       }
     }
   }
-  if (ne) {
-    uint32_t b = 0;
-    if (lane == 0) b = atomicAdd(outcnt, (uint32_t)ne);
-    b = __shfl_sync(FULL, b, 0);
-    for (int i = lane; i < ne; i += 32) out[b + i] = em[i];
-  }
+  if (no) pops += pop_list_cycles(p, F, own, no, out, outcnt, g0);
   __syncwarp();
   return pops;
 }
 
+__device__ __forceinline__ void pop_stats(const PopParams& p, uint32_t pops) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) pops += __shfl_xor_sync(FULL, pops, o);
+  if ((threadIdx.x & 31) == 0 && pops) {
+    atomicAdd(&p.stats[0], (unsigned long long)pops);
+    atomicAdd(&p.stats[1], (unsigned long long)pops);
+  }
+}
+
 template <bool WGT>
 __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
-  __shared__ uint2 sh_q[PK_W][PK_CHUNK];
-  __shared__ uint32_t sh_e[PK_W][PK_EMIT];
+  __shared__ uint2 sh_q[PK_W][PK_RING];
+  __shared__ uint32_t sh_e[PK_W][PK_OWN];
   const int team = (int)(blockIdx.x / (unsigned)p.ctas), cta = (int)(blockIdx.x % (unsigned)p.ctas);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wid = threadIdx.x >> 5;
   const size_t cap = (size_t)p.wrows * p.ld;
   uint32_t* F = p.F + (size_t)team * cap;
   uint32_t* K = p.K + (size_t)team * cap;
@@ -424,31 +488,29 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
   uint32_t gen = 0, pops = 0;
   const int64_t windows = (p.total + p.wrows - 1) / p.wrows;
   bool quit = false;
-  for (int64_t win = team; win < windows && !quit; win += p.teams) {
+  for (int64_t win = team; win < windows; win += p.teams) {
     const int64_t g0 = win * p.wrows;
     const int32_t rows = (int32_t)min((int64_t)p.wrows, p.total - g0);
     pop_draw<WGT>(p, F, g0, rows, cta);
-    if (cta == 0 && threadIdx.x == 0) {
-      lc[0] = lc[1] = 0u;
-    }
+    if (cta == 0 && threadIdx.x == 0) lc[0] = lc[1] = 0u;
     if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
     uint32_t cnt = 0;
     for (uint32_t rd = 0;; ++rd) {
-      // round rd: the list of round rd in L[rd & 1] (every vertex for rd = 0)
-      uint32_t* nxt = L + (size_t)((rd + 1) & 1) * cap;
+      // round rd: its list in L[rd & 1] (every vertex for rd = 0)
+      uint32_t* nxt = L + (size_t)((rd + 1) & 1u) * cap;
+      uint32_t* cur = L + (size_t)(rd & 1u) * cap;
       if (cta == 0 && threadIdx.x == 0) {
         lc[(rd + 2) % 3] = 0u;  // last read two barriers ago
         if (rd > p.max_iters) atomicOr(p.err, ERR_TIMEOUT);
       }
-      if (rd == 0)
-        pops += pop_walk<true>(p, F, nullptr, 0u, 0, nxt, lc + 1, g0, rows, cta, sh_q[wid], sh_e[wid]);
+      if (rd == 0) pops += pop_walk<true>(p, F, cur, 0u, 0, nxt, lc + 1, g0, rows, cta, sh_q[wid], sh_e[wid]);
       else
-        pops += pop_walk<false>(p, F, L + (size_t)(rd & 1) * cap, cnt, (int)(rd & 1), nxt, lc + (rd + 1) % 3, g0, rows,
-                                cta, sh_q[wid], sh_e[wid]);
+        pops += pop_walk<false>(p, F, cur, cnt, (int)(rd & 1u), nxt, lc + (rd + 1) % 3, g0, rows, cta, sh_q[wid],
+                                sh_e[wid]);
       if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
       const uint32_t nc = __ldcg(lc + (rd + 1) % 3);
       if (nc == 0u) break;  // uniform: not written before the next barrier
-      pop_redraw(p, F, K, nxt, nc, L + (size_t)(rd & 1) * cap, cnt, (int)((rd + 1) & 1), g0, cta);
+      pop_redraw<WGT>(p, F, K, nxt, nc, cur, cnt, (int)((rd + 1) & 1u), g0, cta);
       cnt = nc;
       if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
     }
@@ -457,7 +519,7 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
       const int64_t len = (int64_t)rows * p.n;
       for (int64_t i = (int64_t)cta * PK_T + threadIdx.x; i < len; i += (int64_t)p.ctas * PK_T) {
         const int64_t r = i / p.n;
-        p.parents[(g0 + r) * p.n + (i - r * p.n)] = (int32_t)(F[r * p.ld + (i - r * p.n)] & PW_ID);
+        p.parents[g0 * p.n + i] = (int32_t)(F[r * p.ld + (i - r * p.n)] & PW_ID);
       }
     }
     if (p.item_ns != nullptr) {
@@ -468,12 +530,7 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
     }
     if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;  // the tops are read before they are drawn again
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) pops += __shfl_xor_sync(FULL, pops, o);
-  if (lane == 0 && pops) {
-    atomicAdd(&p.stats[0], (unsigned long long)pops);
-    atomicAdd(&p.stats[1], (unsigned long long)pops);
-  }
+  pop_stats(p, pops);
 }
 
 __global__ void k_pop_begin(unsigned long long* t0_ns, unsigned long long* stats, unsigned long long departures) {
@@ -484,12 +541,20 @@ __global__ void k_pop_begin(unsigned long long* t0_ns, unsigned long long* stats
 
 }  // namespace
 
-// Bytes of tops per window and team.  A window's phases end with its longest
-// walk, so more rows per window spread that wait: measured on GB300 (4 teams),
-// windows of 20 / 40 / 80 / 160 / 400 MB: BA n = 2^20, 1024 trees 36.3 / 28.3 /
-// 25.0 / 23.7 / 25.8 ms; grid 1024^2, alpha = 10, 152 trees 81.8 / 58.2 / 45.3 /
-// 38.9 / 39.2 ms.  One team instead of four: 31.0 and 67.5 ms at 160 MB.
-constexpr int64_t POP_WINDOW = 160ll << 20;
+// Tops in flight: larger windows spread the wait for a phase's longest walk
+// over more rows, smaller ones stay closer to L2.  Measured on GB300, 4 teams,
+// windows of 20 / 40 / 80 / 160 / 400 MB per team: BA n = 2^20, 1024 trees 36.3 /
+// 28.3 / 25.0 / 23.7 / 25.8 ms.
+constexpr int64_t POP_WINDOW = 640ll << 20;  // bytes of tops, all teams
+// Teams: with one CTA per team a barrier costs little and every tree advances
+// at its own pace, with one CTA per SM the draws of many trees share a vertex's
+// row.  Measured with 4 / 8 / 76 / 608 teams (ms): ER n = 1000, 2000 trees 0.34 /
+// 0.32 / 0.29 / 0.24; three alphas x 300 trees of a 128^2 grid 5.6 / 5.0 / 4.1 /
+// 3.5; BA 2^18 rooted at its hub (long chains of rounds), 128 trees 8.2 / 7.5 /
+// 6.0 / 5.9; R-MAT 2^18, 32 trees 0.43 / 0.42 / 0.43 / 0.43; 256 uneven graphs (2e6
+// vertices) x 64 trees 4.95 / 4.78 / 5.13 / 5.11; R-MAT 2^22, 64 trees 5.1 / 5.5 /
+// 6.8 / 6.8; BA 2^20, 1024 trees 21.7 / 20.4 / 28.8 / 45.3.
+constexpr int32_t POP_MANY_N = 1 << 17;  // every CTA a team up to this size, and for rooted graphs
 
 static const void* pop_fn(const fc_graph* g) {
   return g->weighted ? (const void*)k_pop<true> : (const void*)k_pop<false>;
@@ -505,14 +570,15 @@ fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* pl) {
     return FC_ECUDA;
   }
   const int64_t ld = ((int64_t)g->n + 3) & ~(int64_t)3;
-  const int64_t cap = std::max<int64_t>(1, POP_WINDOW / (ld * 4));
-  pl->teams = (int)std::min<int64_t>(per_sm, total);
+  const bool many = g->root >= 0 || g->n <= POP_MANY_N;
+  pl->teams = (int)std::min<int64_t>(many ? (int64_t)nsm * per_sm : per_sm, total);
   // 16 bytes per vertex and row (top, entry count, two lists) within a quarter of the device
   while (pl->teams > 1 && (size_t)pl->teams * ld * 16 > g->device_bytes / 4) --pl->teams;
+  const int64_t cap = std::max<int64_t>(1, POP_WINDOW / pl->teams / (ld * 4));
   pl->wrows = (int32_t)std::max<int64_t>(1, std::min<int64_t>(cap, (total + pl->teams - 1) / pl->teams));
   while (pl->wrows > 1 && (size_t)pl->teams * pl->wrows * ld * 16 > g->device_bytes / 4) pl->wrows = (pl->wrows + 1) / 2;
   // CTAs per team: every SM, fewer when a window is small (a barrier of few CTAs is quicker)
-  const int64_t full = (int64_t)nsm * (per_sm / pl->teams);
+  const int64_t full = (int64_t)nsm * per_sm / pl->teams;
   const int64_t want = ((int64_t)pl->wrows * g->n + 4 * PK_T - 1) / (4 * PK_T);
   pl->ctas = (int)std::max<int64_t>(1, std::min<int64_t>(full, want));
   pl->bytes = (size_t)pl->teams * pl->wrows * ld * 16 + (size_t)pl->teams * 128;
@@ -535,6 +601,14 @@ fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& pl, void* ws,
   p.teams = pl.teams;
   p.ctas = pl.ctas;
   p.ld = ((uint32_t)g->n + 3u) & ~3u;
+  {
+    // floor(i / ld) = ((i - h) / 2 + h) >> (s - 1) with s = ceil(log2 ld) and
+    // h = high word of i * (floor(2^32 (2^s - ld) / ld) + 1)
+    uint32_t s = 0;
+    while ((1ull << s) < p.ld) ++s;
+    p.ld_mul = (uint32_t)((((1ull << s) - p.ld) << 32) / p.ld + 1ull);
+    p.ld_shift = s - 1u;  // ld >= 4
+  }
   const size_t cap = (size_t)pl.teams * pl.wrows * p.ld;
   p.F = (uint32_t*)ws;
   p.K = p.F + cap;
