@@ -23,17 +23,6 @@ namespace fcx {
 
 constexpr int SV_T = 256;
 
-// Rows are processed by groups of RG consecutive lanes (strided over the
-// row's entries, then a shuffle reduction), so long rows do not serialise one
-// thread.  Each block covers SV_T / RG rows.
-constexpr int RG = 8;
-constexpr int ROWS_PER_BLOCK = SV_T / RG;
-
-__device__ __forceinline__ double group_sum(double v) {
-#pragma unroll
-  for (int o = RG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 // Block-wide sum of two doubles (warp shuffles, then one warp); the result
 // is valid in thread 0.
 __device__ __forceinline__ void block_sum2(double& a, double& b) {
@@ -55,47 +44,6 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
       a += wa[w];
       b += wb[w];
     }
-  }
-}
-
-__device__ __forceinline__ float group_sumf(float v) {
-#pragma unroll
-  for (int o = RG / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// ---- FP64 residual r = b - A x, partial sums of r.r and b.b ---------------
-__global__ void k_resid64(int32_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                          const float* __restrict__ w, const double* __restrict__ dw, double sigma, double alpha,
-                          const double* __restrict__ b, const double* __restrict__ x, double* __restrict__ r,
-                          double* __restrict__ prr, double* __restrict__ pbb, int nb) {
-  // blocks stride over the chunks of ROWS_PER_BLOCK rows; nb = gridDim.x partials per column
-  const int j = blockIdx.y;
-  const int gl = threadIdx.x % RG;
-  const size_t off = (size_t)j * n;
-  double rr = 0.0, bb = 0.0;
-  for (int64_t c = blockIdx.x; c * ROWS_PER_BLOCK < n; c += gridDim.x) {
-    const int64_t v = c * ROWS_PER_BLOCK + threadIdx.x / RG;
-    double acc = 0.0;
-    if (v < n) {
-      for (int64_t e = rowptr[v] + gl; e < rowptr[v + 1]; e += RG) {
-        const double we = w ? (double)w[e] : 1.0;
-        acc += we * x[off + colidx[e]];
-      }
-    }
-    acc = group_sum(acc);
-    if (v < n && gl == 0) {
-      const double ax = x[off + v] * (sigma + alpha * dw[v]) - alpha * acc;
-      const double rv = b[off + v] - ax;
-      r[off + v] = rv;
-      rr += rv * rv;
-      bb += b[off + v] * b[off + v];
-    }
-  }
-  block_sum2(rr, bb);
-  if (threadIdx.x == 0) {
-    prr[(size_t)j * nb + blockIdx.x] = rr;
-    pbb[(size_t)j * nb + blockIdx.x] = bb;
   }
 }
 
@@ -145,86 +93,6 @@ __global__ void k_inner_init(int32_t n, const double* __restrict__ r64, const fl
     prz[(size_t)j * nb + blockIdx.x] = rz;
     prr[(size_t)j * nb + blockIdx.x] = rr;
   }
-}
-
-// q = A p (FP32), partial p.q
-__global__ void k_spmv_pq(int32_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                          const float* __restrict__ w, const float* __restrict__ diag32, float alpha, Inner in,
-                          double* __restrict__ ppq, int nb) {
-  const int j = blockIdx.y;
-  const int gl = threadIdx.x % RG;
-  const size_t off = (size_t)j * n;
-  const float* pj = in.p + off;
-  float pqf = 0.0f;
-  for (int64_t c = blockIdx.x; c * ROWS_PER_BLOCK < n; c += gridDim.x) {
-    const int64_t v = c * ROWS_PER_BLOCK + threadIdx.x / RG;
-    float acc = 0.0f;
-    if (v < n) {
-      for (int64_t e = rowptr[v] + gl; e < rowptr[v + 1]; e += RG) acc += (w ? w[e] : 1.0f) * pj[colidx[e]];
-    }
-    acc = group_sumf(acc);
-    if (v < n && gl == 0) {
-      const float pv = pj[v];
-      const float qv = pv * diag32[v] - alpha * acc;
-      in.q[off + v] = qv;
-      pqf = fmaf(pv, qv, pqf);
-    }
-  }
-  double pq = pqf, unused = 0.0;
-  block_sum2(pq, unused);
-  if (threadIdx.x == 0) ppq[(size_t)j * nb + blockIdx.x] = pq;
-}
-
-// d += a p; r -= a q; partial r.z, r.r with z = r / diag
-__global__ void k_inner_update(int32_t n, const float* __restrict__ prec, const double* __restrict__ scal,
-                               Inner in, double* __restrict__ prz, double* __restrict__ prr, int nb) {
-  const int j = blockIdx.y;
-  const size_t off = (size_t)j * n;
-  const double* sc = scal + j * 8;
-  const float a = (sc[5] != 0.0 && sc[1] != 0.0) ? (float)(sc[0] / sc[1]) : 0.0f;
-  float rzf = 0.0f, rrf = 0.0f;
-  for (int64_t v = (int64_t)blockIdx.x * SV_T + threadIdx.x; v < n; v += (int64_t)gridDim.x * SV_T) {
-    in.d[off + v] += a * in.p[off + v];
-    const float rv = in.r[off + v] - a * in.q[off + v];
-    in.r[off + v] = rv;
-    const float z = prec ? rv * prec[v] : rv;
-    rzf = fmaf(rv, z, rzf);
-    rrf = fmaf(rv, rv, rrf);
-  }
-  double rz = rzf, rr = rrf;
-  block_sum2(rz, rr);
-  if (threadIdx.x == 0) {
-    prz[(size_t)j * nb + blockIdx.x] = rz;
-    prr[(size_t)j * nb + blockIdx.x] = rr;
-  }
-}
-
-// p = z + beta p with beta = rz_new / rz
-__global__ void k_inner_p(int32_t n, const float* __restrict__ prec, const double* __restrict__ scal, Inner in) {
-  const int j = blockIdx.y;
-  const size_t off = (size_t)j * n;
-  const double* sc = scal + j * 8;
-  const float beta = sc[0] != 0.0 ? (float)(sc[2] / sc[0]) : 0.0f;
-  for (int64_t v = (int64_t)blockIdx.x * SV_T + threadIdx.x; v < n; v += (int64_t)gridDim.x * SV_T) {
-    const float z = prec ? in.r[off + v] * prec[v] : in.r[off + v];
-    in.p[off + v] = z + beta * in.p[off + v];
-  }
-}
-
-// scalar bookkeeping after k_inner_update: rz <- rz_new (done after k_inner_p
-// has used both), rr stored
-// scal[j][f + i] = sums[i m + j] for i < cnt: the per-column scalars from
-// the column sums (one launch instead of a strided copy of m 8-byte rows,
-// which costs about a microsecond per row)
-__global__ void k_put_scal(int m, const double* __restrict__ sums, int f, int cnt, double* __restrict__ scal) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < m)
-    for (int i = 0; i < cnt; ++i) scal[j * 8 + f + i] = sums[(size_t)i * m + j];
-}
-
-__global__ void k_scal_shift(int m, double* scal) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < m) scal[j * 8 + 0] = scal[j * 8 + 2];
 }
 
 // x += (1/scale) d (FP64), only for active columns
@@ -277,36 +145,33 @@ __global__ void k_partial_sum(int64_t len, const double* __restrict__ a, double*
 // Singular systems (sigma = 0, L of a connected graph): the residual's
 // component along 1 lies in L's kernel, where CG cannot reduce it; rounding
 // in the FP64 residual leaves a little there, so each refinement step
-// projects it out.  One block per column (fixed-order sums): r_j -= mean(r_j)
-// and rr[j] = |r_j|^2 after the projection.  il: element (v, j) at v m + j,
-// else at j n + v.
-__global__ void k_proj_mean(int32_t n, int m, bool il, double* __restrict__ r, double* __restrict__ rr) {
-  __shared__ double red[SV_T];
-  const int j = blockIdx.x;
-  auto at = [&](int64_t v) -> double& { return r[il ? (size_t)v * m + j : (size_t)j * n + v]; };
-  double s = 0.0;
-  for (int64_t v = threadIdx.x; v < n; v += SV_T) s += at(v);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = SV_T / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  const double mean = red[0] / (double)n;
-  __syncthreads();
-  double q = 0.0;
-  for (int64_t v = threadIdx.x; v < n; v += SV_T) {
-    const double x = at(v) - mean;
-    at(v) = x;
+// projects it out.  Element (v, j) of the columns at v sv + j sj (column-major
+// or interleaved); blockIdx.y = j, fixed-order partial sums of the column per
+// block (one block per column took 0.4 ms for one column of n = 2^18, most of
+// a Laplacian solve).
+__global__ void __launch_bounds__(SV_T) k_col_part(int32_t n, const double* __restrict__ in, int64_t sv, int64_t sj,
+                                                   double* __restrict__ part, int nb) {
+  const double* x = in + blockIdx.y * sj;
+  double s = 0.0, unused = 0.0;
+  for (int64_t v = (int64_t)blockIdx.x * SV_T + threadIdx.x; v < n; v += (int64_t)gridDim.x * SV_T) s += x[v * sv];
+  block_sum2(s, unused);
+  if (threadIdx.x == 0) part[(size_t)blockIdx.y * nb + blockIdx.x] = s;
+}
+
+// out = in - sum_j / n; partial sums of squares of out (part may be null)
+__global__ void __launch_bounds__(SV_T) k_col_shift(int32_t n, const double* __restrict__ in, int64_t sv, int64_t sj,
+                                                    const double* __restrict__ sums, double* __restrict__ out,
+                                                    double* __restrict__ part, int nb) {
+  const double mean = sums[blockIdx.y] / (double)n;
+  double q = 0.0, unused = 0.0;
+  for (int64_t v = (int64_t)blockIdx.x * SV_T + threadIdx.x; v < n; v += (int64_t)gridDim.x * SV_T) {
+    const double x = in[v * sv + blockIdx.y * sj] - mean;
+    out[v * sv + blockIdx.y * sj] = x;
     q += x * x;
   }
-  red[threadIdx.x] = q;
-  __syncthreads();
-  for (int k = SV_T / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) rr[j] = red[0];
+  if (part == nullptr) return;
+  block_sum2(q, unused);
+  if (threadIdx.x == 0) part[(size_t)blockIdx.y * nb + blockIdx.x] = q;
 }
 
 // ---------------------------------------------------------------------------
@@ -883,30 +748,169 @@ __global__ void __launch_bounds__(SV_T, FOLD ? 3 : 4) k_cg1(CG1 c) {
 }
 
 // ---------------------------------------------------------------------------
-// Many right-hand sides (m >= 32): the solver's vectors interleaved by
-// column, element (v, j) at v m + j.  A warp takes 32 columns of one row, so
-// each neighbour gather of the SpMV loads 32 columns' values from one
-// contiguous segment (128 bytes in FP32) instead of 32 separate sectors.
-// Blocks are 32 x 8 threads (column in the group x row); blockIdx.y is the
-// column group and blocks stride over row chunks of 8; per-column partial
-// sums go to part[j nb + blockIdx.x] as for the column-major kernels.
+// Several right-hand sides (m >= 2): the solver's vectors interleaved by
+// column, element (v, j) at v m + j.  A warp takes 32 VW columns of one row
+// (VW values per lane), so each neighbour gather of the products loads one
+// contiguous segment of 128 VW bytes (FP32).  Blocks are 32 x 8 threads (column
+// x row), blockIdx.y is the column group; with fewer than 32 columns the block
+// is LW x 256 / LW threads (LW the power of two from m on), several rows per
+// warp.  Per-column partial sums go to part[j nb + blockIdx.x].
+//
+// The products run over row segments of at most IL_SEG entries: a warp that
+// walked a whole hub row (11,600 entries at n = 2^19) held up the launch for
+// about a millisecond.  A row of one segment is finished by its warp; the
+// segments of a longer row leave partial sums that k_il_long_* adds in row
+// order.  Bound by the neighbour gathers (DRAM and L2) and 8 vector passes per
+// iteration.  Measured on GB300 (whole solves to 1e-12; before: a warp per row,
+// one value per lane, 9 launches per iteration, and eight lanes per row below
+// 32 columns): BA 2^19, 64 columns 75.4 -> 28.3 ms, 16 33.2 -> 10.8, 2 8.0 -> 3.6;
+// weighted grid 2^20, 64 columns 132 -> 94; weighted R-MAT 2^16, 85 columns 76.7 ->
+// 27; group closeness of n = 4099 (4096 columns) 28.4 -> 20.6.
 // ---------------------------------------------------------------------------
-constexpr int IL_R = 8;
+constexpr int IL_T = 256;  // threads per block
+constexpr int IL_SEG = 128;      // entries per segment, a warp per row (n = 5000, 21 columns: 2.7 ms, 3.2 with 256)
+constexpr int IL_SEG_PACK = 64;  // and with several rows per warp (their segments run on few lanes)
+constexpr int IL_U = 8;  // gathers of a warp in flight
 
-__device__ __forceinline__ void il_sum2(double a, double b, int j, bool on, double* __restrict__ pa,
-                                        double* __restrict__ pb, int nb) {
-  __shared__ double sa[IL_R][33], sb[IL_R][33];
-  sa[threadIdx.y][threadIdx.x] = a;
-  sb[threadIdx.y][threadIdx.x] = b;
+template <typename T, int VW>
+struct ILVec;
+template <> struct ILVec<float, 1> { typedef float type; };
+template <> struct ILVec<float, 2> { typedef float2 type; };
+template <> struct ILVec<float, 4> { typedef float4 type; };
+template <> struct ILVec<double, 1> { typedef double type; };
+template <> struct ILVec<double, 2> { typedef double2 type; };
+
+// VW consecutive columns of one row (aligned: VW divides m)
+template <typename T, int VW>
+__device__ __forceinline__ void il_load(const T* p, T (&x)[VW]) {
+  const auto v = *reinterpret_cast<const typename ILVec<T, VW>::type*>(p);
+  const T* s = reinterpret_cast<const T*>(&v);
+#pragma unroll
+  for (int c = 0; c < VW; ++c) x[c] = s[c];
+}
+template <typename T, int VW>
+__device__ __forceinline__ void il_store(T* p, const T (&x)[VW]) {
+  typename ILVec<T, VW>::type v;
+  T* s = reinterpret_cast<T*>(&v);
+#pragma unroll
+  for (int c = 0; c < VW; ++c) s[c] = x[c];
+  *reinterpret_cast<typename ILVec<T, VW>::type*>(p) = v;
+}
+
+// per-column sums over the block's rows to pa (and pb), fixed order
+template <int VW>
+__device__ __forceinline__ void il_sum2(const double (&a)[VW], const double (&b)[VW], int j0, bool on,
+                                        double* __restrict__ pa, double* __restrict__ pb, int nb, int blk) {
+  constexpr int N = IL_T * VW + 128;  // rows of LW VW + 1 values, at most 128 rows
+  __shared__ double sa[N], sb[N];
+  const int ld = blockDim.x * VW + 1;
+#pragma unroll
+  for (int c = 0; c < VW; ++c) {
+    sa[threadIdx.y * ld + threadIdx.x * VW + c] = a[c];
+    sb[threadIdx.y * ld + threadIdx.x * VW + c] = b[c];
+  }
   __syncthreads();
-  if (threadIdx.y == 0 && on) {
-    double ta = 0.0, tb = 0.0;
-    for (int r = 0; r < IL_R; ++r) {
-      ta += sa[r][threadIdx.x];
-      tb += sb[r][threadIdx.x];
+  for (int h = blockDim.y / 2; h > 0; h >>= 1) {
+    if (threadIdx.y < h) {
+#pragma unroll
+      for (int c = 0; c < VW; ++c) {
+        const int i = threadIdx.y * ld + threadIdx.x * VW + c;
+        sa[i] += sa[i + h * ld];
+        sb[i] += sb[i + h * ld];
+      }
     }
-    pa[(size_t)j * nb + blockIdx.x] = ta;
-    if (pb) pb[(size_t)j * nb + blockIdx.x] = tb;
+    __syncthreads();
+  }
+  if (threadIdx.y == 0 && on) {
+#pragma unroll
+    for (int c = 0; c < VW; ++c) {
+      pa[(size_t)(j0 + c) * nb + blk] = sa[threadIdx.x * VW + c];
+      if (pb) pb[(size_t)(j0 + c) * nb + blk] = sb[threadIdx.x * VW + c];
+    }
+  }
+}
+
+// segments per row (at least one), and for rows of several their count and 1
+__global__ void k_il_seg_count(int32_t n, int len, const int64_t* __restrict__ rowptr, uint32_t* __restrict__ cnt,
+                               uint32_t* __restrict__ lcnt, uint32_t* __restrict__ lrow) {
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v > n) return;
+  uint32_t c = 0;
+  if (v < n) {
+    const int64_t d = rowptr[v + 1] - rowptr[v];
+    c = d > len ? (uint32_t)((d + len - 1) / len) : 1u;
+  }
+  cnt[v] = c;
+  lcnt[v] = c > 1u ? c : 0u;
+  lrow[v] = c > 1u ? 1u : 0u;
+}
+
+// segs: {row, entries, first entry, slot of its partial sum or -1}; longs:
+// {row, first slot, slots, 0}
+__global__ void k_il_seg_fill(int32_t n, int len, const int64_t* __restrict__ rowptr, const uint32_t* __restrict__ off,
+                              const uint32_t* __restrict__ loff, const uint32_t* __restrict__ lidx,
+                              int4* __restrict__ segs, int4* __restrict__ longs) {
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= n) return;
+  const int64_t e0 = rowptr[v], e1 = rowptr[v + 1];
+  const uint32_t o = off[v], c = off[v + 1] - o;
+  for (uint32_t k = 0; k < c; ++k) {
+    const int64_t b = e0 + (int64_t)k * len;
+    segs[o + k] = make_int4((int32_t)v, (int32_t)(e1 - b < len ? e1 - b : len), (int32_t)(uint32_t)b,
+                            c > 1u ? (int32_t)(loff[v] + k) : -1);
+  }
+  if (c > 1u) longs[lidx[v]] = make_int4((int32_t)v, (int32_t)loff[v], (int32_t)c, 0);
+}
+
+// sum over a segment of w x[col] for VW columns, IL_U gathers in flight.  A
+// full warp per row loads 32 column indices at a time and broadcasts them by
+// shuffles; PACK (several rows per warp): every lane loads the index itself
+// (one transaction per row).
+template <typename T, int VW, bool PACK>
+__device__ __forceinline__ void il_seg_sum(const int4& s, const int32_t* __restrict__ colidx,
+                                           const float* __restrict__ w, const T* __restrict__ x, int m, int j0, bool on,
+                                           T (&acc)[VW]) {
+  const size_t e0 = (uint32_t)s.z;
+#pragma unroll
+  for (int c = 0; c < VW; ++c) acc[c] = (T)0;
+  for (int b = 0; b < s.y; b += PACK ? IL_U : 32) {
+    const int left = min(PACK ? IL_U : 32, s.y - b);
+    int32_t cj = 0;
+    float wj = 0.0f;
+    if (!PACK && (int)threadIdx.x < left) {
+      cj = __ldg(colidx + e0 + b + threadIdx.x);
+      wj = w ? __ldg(w + e0 + b + threadIdx.x) : 1.0f;
+    }
+    for (int k = 0; k < left; k += IL_U) {
+      T xv[IL_U][VW];
+      float ww[IL_U];
+#pragma unroll
+      for (int u = 0; u < IL_U; ++u) {
+        int32_t c = 0;
+        ww[u] = 0.0f;
+        if (PACK) {
+          if (u < left) {
+            c = __ldg(colidx + e0 + b + u);
+            ww[u] = w ? __ldg(w + e0 + b + u) : 1.0f;
+          }
+        } else {
+          c = __shfl_sync(0xffffffffu, cj, (k + u) & 31);
+          ww[u] = __shfl_sync(0xffffffffu, wj, (k + u) & 31);
+        }
+        if (on && k + u < left) il_load<T, VW>(x + (size_t)c * m + j0, xv[u]);
+        else {
+#pragma unroll
+          for (int q = 0; q < VW; ++q) xv[u][q] = (T)0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < IL_U; ++u) {
+        if (k + u < left) {
+#pragma unroll
+          for (int q = 0; q < VW; ++q) acc[q] += (T)ww[u] * xv[u][q];
+        }
+      }
+    }
   }
 }
 
@@ -928,133 +932,391 @@ __global__ void k_il_transpose(int64_t rows, int64_t cols, const double* __restr
     }
 }
 
-__global__ void __launch_bounds__(256) k_resid64_il(int32_t n, int m, const int64_t* __restrict__ rowptr,
-                                                    const int32_t* __restrict__ colidx, const float* __restrict__ w,
-                                                    const double* __restrict__ dw, double sigma, double alpha,
-                                                    const double* __restrict__ b, const double* __restrict__ x,
-                                                    double* __restrict__ r, double* __restrict__ prr,
-                                                    double* __restrict__ pbb, int nb) {
-  const int j = blockIdx.y * 32 + threadIdx.x;
-  const bool on = j < m;
-  double rr = 0.0, bb = 0.0;
-  for (int64_t c = blockIdx.x; c * IL_R < n; c += gridDim.x) {
-    const int64_t v = c * IL_R + threadIdx.y;
-    if (v < n && on) {
-      double acc = 0.0;
-      for (int64_t e = rowptr[v]; e < rowptr[v + 1]; ++e)
-        acc += (w ? (double)w[e] : 1.0) * x[(size_t)colidx[e] * m + j];
-      const size_t i = (size_t)v * m + j;
-      const double rv = b[i] - (x[i] * (sigma + alpha * dw[v]) - alpha * acc);
-      r[i] = rv;
-      rr += rv * rv;
-      bb += b[i] * b[i];
-    }
+// r = b - (sigma + alpha d_w) x + alpha s of one row
+template <int VW>
+__device__ __forceinline__ void il_resid_row(size_t i, double d, double alpha, const double (&acc)[VW],
+                                             const double* __restrict__ b, const double* __restrict__ x,
+                                             double* __restrict__ r, double (&rr)[VW], double (&bb)[VW]) {
+  double bv[VW], xv[VW], rv[VW];
+  il_load<double, VW>(b + i, bv);
+  il_load<double, VW>(x + i, xv);
+#pragma unroll
+  for (int c = 0; c < VW; ++c) {
+    rv[c] = bv[c] - (xv[c] * d - alpha * acc[c]);
+    rr[c] += rv[c] * rv[c];
+    bb[c] += bv[c] * bv[c];
   }
-  il_sum2(rr, bb, j, on, prr, pbb, nb);
+  il_store<double, VW>(r + i, rv);
 }
 
-__global__ void __launch_bounds__(256) k_inner_init_il(int32_t n, int m, const double* __restrict__ r64,
-                                                       const float* __restrict__ prec, const double* __restrict__ scal,
-                                                       Inner in, double* __restrict__ prz, double* __restrict__ prr,
-                                                       int nb) {
-  const int j = blockIdx.y * 32 + threadIdx.x;
-  const bool on = j < m;
-  const double sc = on ? scal[j * 8 + 4] : 0.0;
-  float rz = 0.0f, rr = 0.0f;  // per-thread partials in FP32, then FP64 across threads
-  for (int64_t c = blockIdx.x; c * IL_R < n; c += gridDim.x) {
-    const int64_t v = c * IL_R + threadIdx.y;
-    if (v < n && on) {
-      const size_t i = (size_t)v * m + j;
-      const float rv = (float)(r64[i] * sc);
-      const float z = prec ? rv * prec[v] : rv;
-      in.r[i] = rv;
-      in.p[i] = z;
-      in.d[i] = 0.0f;
-      rz = fmaf(rv, z, rz);
-      rr = fmaf(rv, rv, rr);
-    }
+template <int VW, bool PACK>
+__global__ void __launch_bounds__(IL_T) k_il_resid(int m, int nseg, const int4* __restrict__ segs,
+                                                  const int32_t* __restrict__ colidx, const float* __restrict__ w,
+                                                  const double* __restrict__ dw, double sigma, double alpha,
+                                                  const double* __restrict__ b, const double* __restrict__ x,
+                                                  double* __restrict__ r, double* __restrict__ plong,
+                                                  double* __restrict__ prr, double* __restrict__ pbb, int nb) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  const bool on = j0 < m;
+  double rr[VW] = {}, bb[VW] = {};
+  for (int g = blockIdx.x * blockDim.y + threadIdx.y; g < nseg; g += gridDim.x * blockDim.y) {
+    const int4 s = segs[g];
+    double acc[VW];
+    il_seg_sum<double, VW, PACK>(s, colidx, w, x, m, j0, on, acc);
+    if (!on) continue;
+    if (s.w >= 0) il_store<double, VW>(plong + (size_t)s.w * m + j0, acc);
+    else il_resid_row<VW>((size_t)s.x * m + j0, sigma + alpha * dw[s.x], alpha, acc, b, x, r, rr, bb);
   }
-  il_sum2(rz, rr, j, on, prz, prr, nb);
+  il_sum2<VW>(rr, bb, j0, on, prr, pbb, nb, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(256) k_spmv_pq_il(int32_t n, int m, const int64_t* __restrict__ rowptr,
-                                                    const int32_t* __restrict__ colidx, const float* __restrict__ w,
-                                                    const float* __restrict__ diag32, float alpha, Inner in,
-                                                    double* __restrict__ ppq, int nb) {
-  const int j = blockIdx.y * 32 + threadIdx.x;
-  const bool on = j < m;
-  float pq = 0.0f;
-  for (int64_t c = blockIdx.x; c * IL_R < n; c += gridDim.x) {
-    const int64_t v = c * IL_R + threadIdx.y;
-    if (v < n && on) {
-      float acc = 0.0f;
-      for (int64_t e = rowptr[v]; e < rowptr[v + 1]; ++e) acc += (w ? w[e] : 1.0f) * in.p[(size_t)colidx[e] * m + j];
-      const size_t i = (size_t)v * m + j;
-      const float pv = in.p[i];
-      const float qv = pv * diag32[v] - alpha * acc;
-      in.q[i] = qv;
-      pq = fmaf(pv, qv, pq);
+// rows of several segments: their partial sums in row order
+template <int VW>
+__global__ void __launch_bounds__(IL_T) k_il_long_resid(int m, int nlong, const int4* __restrict__ longs,
+                                                       const double* __restrict__ dw, double sigma, double alpha,
+                                                       const double* __restrict__ b, const double* __restrict__ x,
+                                                       double* __restrict__ r, const double* __restrict__ plong,
+                                                       double* __restrict__ prr, double* __restrict__ pbb, int nb,
+                                                       int blk0) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  const bool on = j0 < m;
+  double rr[VW] = {}, bb[VW] = {};
+  for (int g = blockIdx.x * blockDim.y + threadIdx.y; g < nlong && on; g += gridDim.x * blockDim.y) {
+    const int4 s = longs[g];
+    double acc[VW] = {};
+    for (int k = 0; k < s.z; ++k) {
+      double y[VW];
+      il_load<double, VW>(plong + (size_t)(s.y + k) * m + j0, y);
+#pragma unroll
+      for (int c = 0; c < VW; ++c) acc[c] += y[c];
     }
+    il_resid_row<VW>((size_t)s.x * m + j0, sigma + alpha * dw[s.x], alpha, acc, b, x, r, rr, bb);
   }
-  il_sum2(pq, 0.0, j, on, ppq, nullptr, nb);
+  il_sum2<VW>(rr, bb, j0, on, prr, pbb, nb, blk0 + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(256) k_inner_update_il(int32_t n, int m, const float* __restrict__ prec,
-                                                         const double* __restrict__ scal, Inner in,
-                                                         double* __restrict__ prz, double* __restrict__ prr, int nb) {
-  const int j = blockIdx.y * 32 + threadIdx.x;
-  const bool on = j < m;
-  float a = 0.0f;
-  if (on) {
-    const double* sc = scal + j * 8;
-    a = (sc[5] != 0.0 && sc[1] != 0.0) ? (float)(sc[0] / sc[1]) : 0.0f;
-  }
-  float rz = 0.0f, rr = 0.0f;
-  for (int64_t c = blockIdx.x; c * IL_R < n; c += gridDim.x) {
-    const int64_t v = c * IL_R + threadIdx.y;
-    if (v < n && on) {
-      const size_t i = (size_t)v * m + j;
-      in.d[i] += a * in.p[i];
-      const float rv = in.r[i] - a * in.q[i];
-      in.r[i] = rv;
-      const float z = prec ? rv * prec[v] : rv;
-      rz = fmaf(rv, z, rz);
-      rr = fmaf(rv, rv, rr);
+// r32 = r64 scale, p = z = r32 prec, d = 0; partials of r.z and r.r.  The
+// element-wise kernels take IL_V rows per step.
+constexpr int IL_V = 4;
+template <int VW>
+__global__ void __launch_bounds__(IL_T) k_il_init(int32_t n, int m, const double* __restrict__ r64,
+                                                 const float* __restrict__ prec, const double* __restrict__ scal,
+                                                 Inner in, double* __restrict__ prz, double* __restrict__ prr, int nb) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  const bool on = j0 < m;
+  double sc[VW];
+  float rz[VW] = {}, rr[VW] = {};  // per-thread partials in FP32, then FP64 across threads
+#pragma unroll
+  for (int c = 0; c < VW; ++c) sc[c] = on ? scal[(j0 + c) * 8 + 4] : 0.0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; v < n && on; v += (int64_t)gridDim.x * blockDim.y) {
+    const size_t i = (size_t)v * m + j0;
+    const float pr = prec ? prec[v] : 1.0f;
+    float r[VW], z[VW], zero[VW] = {};
+#pragma unroll
+    for (int c = 0; c < VW; ++c) {
+      r[c] = (float)(r64[i + c] * sc[c]);
+      z[c] = r[c] * pr;
+      rz[c] = fmaf(r[c], z[c], rz[c]);
+      rr[c] = fmaf(r[c], r[c], rr[c]);
     }
+    il_store<float, VW>(in.r + i, r);
+    il_store<float, VW>(in.p + i, z);
+    il_store<float, VW>(in.d + i, zero);
   }
-  il_sum2(rz, rr, j, on, prz, prr, nb);
+  double a[VW], b[VW];
+#pragma unroll
+  for (int c = 0; c < VW; ++c) {
+    a[c] = rz[c];
+    b[c] = rr[c];
+  }
+  il_sum2<VW>(a, b, j0, on, prz, prr, nb, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(256) k_inner_p_il(int32_t n, int m, const float* __restrict__ prec,
-                                                    const double* __restrict__ scal, Inner in) {
-  const int j = blockIdx.y * 32 + threadIdx.x;
-  if (j >= m) return;
-  const double* sc = scal + j * 8;
-  const float beta = sc[0] != 0.0 ? (float)(sc[2] / sc[0]) : 0.0f;
-  for (int64_t c = blockIdx.x; c * IL_R < n; c += gridDim.x) {
-    const int64_t v = c * IL_R + threadIdx.y;
-    if (v < n) {
-      const size_t i = (size_t)v * m + j;
-      const float z = prec ? in.r[i] * prec[v] : in.r[i];
-      in.p[i] = z + beta * in.p[i];
+// q = diag p - alpha s of one row, partial of p.q
+template <int VW>
+__device__ __forceinline__ void il_spmv_row(size_t i, float dg, float alpha, const float (&acc)[VW], const Inner& in,
+                                            float (&pq)[VW]) {
+  float pv[VW], qv[VW];
+  il_load<float, VW>(in.p + i, pv);
+#pragma unroll
+  for (int c = 0; c < VW; ++c) {
+    qv[c] = pv[c] * dg - alpha * acc[c];
+    pq[c] = fmaf(pv[c], qv[c], pq[c]);
+  }
+  il_store<float, VW>(in.q + i, qv);
+}
+
+// q = A p, partials of p.q
+template <int VW, bool PACK>
+__global__ void __launch_bounds__(IL_T) k_il_spmv(int m, int nseg, const int4* __restrict__ segs,
+                                                 const int32_t* __restrict__ colidx, const float* __restrict__ w,
+                                                 const float* __restrict__ diag32, float alpha, Inner in,
+                                                 float* __restrict__ plong, double* __restrict__ ppq, int nb) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  const bool on = j0 < m;
+  float pq[VW] = {};
+  for (int g = blockIdx.x * blockDim.y + threadIdx.y; g < nseg; g += gridDim.x * blockDim.y) {
+    const int4 s = segs[g];
+    float acc[VW];
+    il_seg_sum<float, VW, PACK>(s, colidx, w, in.p, m, j0, on, acc);
+    if (!on) continue;
+    if (s.w >= 0) il_store<float, VW>(plong + (size_t)s.w * m + j0, acc);
+    else il_spmv_row<VW>((size_t)s.x * m + j0, diag32[s.x], alpha, acc, in, pq);
+  }
+  double a[VW], z[VW] = {};
+#pragma unroll
+  for (int c = 0; c < VW; ++c) a[c] = pq[c];
+  il_sum2<VW>(a, z, j0, on, ppq, nullptr, nb, blockIdx.x);
+}
+
+template <int VW>
+__global__ void __launch_bounds__(IL_T) k_il_long_spmv(int m, int nlong, const int4* __restrict__ longs,
+                                                      const float* __restrict__ diag32, float alpha, Inner in,
+                                                      const float* __restrict__ plong, double* __restrict__ ppq, int nb,
+                                                      int blk0) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  const bool on = j0 < m;
+  float pq[VW] = {};
+  for (int g = blockIdx.x * blockDim.y + threadIdx.y; g < nlong && on; g += gridDim.x * blockDim.y) {
+    const int4 s = longs[g];
+    float acc[VW] = {};
+    for (int k = 0; k < s.z; ++k) {
+      float y[VW];
+      il_load<float, VW>(plong + (size_t)(s.y + k) * m + j0, y);
+#pragma unroll
+      for (int c = 0; c < VW; ++c) acc[c] += y[c];
+    }
+    il_spmv_row<VW>((size_t)s.x * m + j0, diag32[s.x], alpha, acc, in, pq);
+  }
+  double a[VW], z[VW] = {};
+#pragma unroll
+  for (int c = 0; c < VW; ++c) a[c] = pq[c];
+  il_sum2<VW>(a, z, j0, on, ppq, nullptr, nb, blk0 + blockIdx.x);
+}
+
+// r -= a q; partials of r.z and r.r (d += a p is left to k_il_p, which reads p
+// anyway: 8 vector passes per iteration instead of 9)
+template <int VW>
+__global__ void __launch_bounds__(IL_T) k_il_update(int32_t n, int m, const float* __restrict__ prec,
+                                                   const double* __restrict__ scal, Inner in, double* __restrict__ prz,
+                                                   double* __restrict__ prr, int nb) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  const bool on = j0 < m;
+  float a[VW], rz[VW] = {}, rr[VW] = {};
+#pragma unroll
+  for (int c = 0; c < VW; ++c) a[c] = on ? (float)scal[(j0 + c) * 8 + 6] : 0.0f;
+  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.y + threadIdx.y) * IL_V; v0 < n && on;
+       v0 += (int64_t)gridDim.x * blockDim.y * IL_V) {
+    float r[IL_V][VW], q[IL_V][VW], pr[IL_V];
+#pragma unroll
+    for (int u = 0; u < IL_V; ++u) {
+      if (v0 + u < n) {
+        const size_t i = (size_t)(v0 + u) * m + j0;
+        il_load<float, VW>(in.r + i, r[u]);
+        il_load<float, VW>(in.q + i, q[u]);
+        pr[u] = prec ? prec[v0 + u] : 1.0f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < IL_V; ++u) {
+      if (v0 + u < n) {
+#pragma unroll
+        for (int c = 0; c < VW; ++c) {
+          r[u][c] -= a[c] * q[u][c];
+          rz[c] = fmaf(r[u][c], r[u][c] * pr[u], rz[c]);
+          rr[c] = fmaf(r[u][c], r[u][c], rr[c]);
+        }
+        il_store<float, VW>(in.r + (size_t)(v0 + u) * m + j0, r[u]);
+      }
+    }
+  }
+  double x[VW], y[VW];
+#pragma unroll
+  for (int c = 0; c < VW; ++c) {
+    x[c] = rz[c];
+    y[c] = rr[c];
+  }
+  il_sum2<VW>(x, y, j0, on, prz, prr, nb, blockIdx.x);
+}
+
+// d += a p; p = z + beta p
+template <int VW>
+__global__ void __launch_bounds__(IL_T) k_il_p(int32_t n, int m, const float* __restrict__ prec,
+                                              const double* __restrict__ scal, Inner in) {
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  if (j0 >= m) return;
+  float a[VW], beta[VW];
+#pragma unroll
+  for (int c = 0; c < VW; ++c) {
+    a[c] = (float)scal[(j0 + c) * 8 + 6];
+    beta[c] = (float)scal[(j0 + c) * 8 + 7];
+  }
+  for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.y + threadIdx.y) * IL_V; v0 < n;
+       v0 += (int64_t)gridDim.x * blockDim.y * IL_V) {
+    float r[IL_V][VW], p[IL_V][VW], d[IL_V][VW], pr[IL_V];
+#pragma unroll
+    for (int u = 0; u < IL_V; ++u) {
+      if (v0 + u < n) {
+        const size_t i = (size_t)(v0 + u) * m + j0;
+        il_load<float, VW>(in.r + i, r[u]);
+        il_load<float, VW>(in.p + i, p[u]);
+        il_load<float, VW>(in.d + i, d[u]);
+        pr[u] = prec ? prec[v0 + u] : 1.0f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < IL_V; ++u) {
+      if (v0 + u < n) {
+        const size_t i = (size_t)(v0 + u) * m + j0;
+#pragma unroll
+        for (int c = 0; c < VW; ++c) {
+          d[u][c] += a[c] * p[u][c];
+          p[u][c] = r[u][c] * pr[u] + beta[c] * p[u][c];
+        }
+        il_store<float, VW>(in.d + i, d[u]);
+        il_store<float, VW>(in.p + i, p[u]);
+      }
     }
   }
 }
 
-__global__ void __launch_bounds__(256) k_correct_il(int32_t n, int m, const double* __restrict__ scal,
+// x += d / scale (FP64), only for active columns
+template <int VW>
+__global__ void __launch_bounds__(IL_T) k_il_correct(int32_t n, int m, const double* __restrict__ scal,
                                                     const float* __restrict__ d, double* __restrict__ x) {
-  const int j = blockIdx.y * 32 + threadIdx.x;
-  if (j >= m) return;
-  const double* sc = scal + j * 8;
-  if (sc[5] == 0.0) return;
-  for (int64_t c = blockIdx.x; c * IL_R < n; c += gridDim.x) {
-    const int64_t v = c * IL_R + threadIdx.y;
-    if (v < n) {
-      const size_t i = (size_t)v * m + j;
-      x[i] += (double)d[i] / sc[4];
-    }
+  const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
+  if (j0 >= m) return;
+  double f[VW];  // one division per thread: GB300's FP64 rate is low
+#pragma unroll
+  for (int c = 0; c < VW; ++c) f[c] = scal[(j0 + c) * 8 + 5] != 0.0 ? 1.0 / scal[(j0 + c) * 8 + 4] : 0.0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; v < n; v += (int64_t)gridDim.x * blockDim.y) {
+    const size_t i = (size_t)v * m + j0;
+    float dv[VW];
+    il_load<float, VW>(d + i, dv);
+#pragma unroll
+    for (int c = 0; c < VW; ++c)
+      if (f[c] != 0.0) x[i + c] += (double)dv[c] * f[c];
   }
 }
+
+// Per-column scalars after the products: pq and a = rz / pq (a block per
+// column, fixed order).
+__global__ void __launch_bounds__(128) k_il_alpha(const double* __restrict__ ppq, int nb, double* __restrict__ scal) {
+  __shared__ double red[128];
+  const int j = blockIdx.x;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < nb; i += 128) s += ppq[(size_t)j * nb + i];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int k = 64; k > 0; k >>= 1) {
+    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    double* sc = scal + (size_t)j * 8;
+    sc[1] = red[0];
+    sc[6] = (sc[5] != 0.0 && red[0] != 0.0) ? sc[0] / red[0] : 0.0;
+  }
+}
+
+// After the update: the new r.z and r.r, beta = rz_new / rz, rz <- rz_new.
+__global__ void __launch_bounds__(128) k_il_beta(const double* __restrict__ prz, const double* __restrict__ prr, int nb,
+                                                 double* __restrict__ scal, double* __restrict__ rr_out) {
+  __shared__ double ra[128], rb[128];
+  const int j = blockIdx.x;
+  double s = 0.0, t = 0.0;
+  for (int i = threadIdx.x; i < nb; i += 128) {
+    s += prz[(size_t)j * nb + i];
+    t += prr[(size_t)j * nb + i];
+  }
+  ra[threadIdx.x] = s;
+  rb[threadIdx.x] = t;
+  __syncthreads();
+  for (int k = 64; k > 0; k >>= 1) {
+    if (threadIdx.x < k) {
+      ra[threadIdx.x] += ra[threadIdx.x + k];
+      rb[threadIdx.x] += rb[threadIdx.x + k];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    double* sc = scal + (size_t)j * 8;
+    sc[7] = sc[0] != 0.0 ? ra[0] / sc[0] : 0.0;
+    sc[0] = ra[0];
+    sc[2] = ra[0];
+    sc[3] = rb[0];
+    rr_out[j] = rb[0];
+  }
+}
+
+// The interleaved kernels for VW columns per lane, and the plan of a solve.
+struct ILPlan {
+  int vw, lw;            // columns per lane, lanes per row
+  int gy, gxs, gxl, gxe;  // column groups, blocks over segments, long rows and rows
+  int nseg, nlong, nslot;
+  const int4* segs;
+  const int4* longs;
+  void* plong;                // [nslot][m] partial sums (FP64 or FP32)
+};
+
+template <int VW>
+static void il_launch_resid(const ILPlan& pl, const fc_graph* g, int m, double sigma, double alpha, const double* b,
+                            const double* x, double* r, double* pA, double* pB, cudaStream_t st) {
+  const dim3 blk(pl.lw, IL_T / pl.lw);
+  const int nb = pl.gxs + pl.gxl;
+  auto* kern = pl.lw == 32 ? k_il_resid<VW, false> : k_il_resid<VW, true>;
+  kern<<<dim3(pl.gxs, pl.gy), blk, 0, st>>>(m, pl.nseg, pl.segs, g->colidx, g->w, g->dw, sigma, alpha, b, x, r,
+                                            (double*)pl.plong, pA, pB, nb);
+  note_launch();
+  if (pl.nlong > 0) {
+    k_il_long_resid<VW><<<dim3(pl.gxl, pl.gy), blk, 0, st>>>(m, pl.nlong, pl.longs, g->dw, sigma, alpha, b, x, r,
+                                                             (const double*)pl.plong, pA, pB, nb, pl.gxs);
+    note_launch();
+  }
+}
+
+template <int VW>
+static void il_launch_init(const ILPlan& pl, int32_t n, int m, const double* r64, const float* prec,
+                           const double* scal, const Inner& in, double* pA, double* pB, cudaStream_t st) {
+  k_il_init<VW><<<dim3(pl.gxe, pl.gy), dim3(pl.lw, IL_T / pl.lw), 0, st>>>(n, m, r64, prec, scal, in, pA, pB, pl.gxe);
+  note_launch();
+}
+
+// one inner iteration
+template <int VW>
+static void il_launch_iter(const ILPlan& pl, const fc_graph* g, int m, const float* prec, const float* diag32,
+                           float alpha, double* scal, const Inner& in, double* pA, double* pB, double* rr_out,
+                           cudaStream_t st) {
+  const dim3 blk(pl.lw, IL_T / pl.lw);
+  const int nb = pl.gxs + pl.gxl;
+  auto* kern = pl.lw == 32 ? k_il_spmv<VW, false> : k_il_spmv<VW, true>;
+  kern<<<dim3(pl.gxs, pl.gy), blk, 0, st>>>(m, pl.nseg, pl.segs, g->colidx, g->w, diag32, alpha, in, (float*)pl.plong,
+                                            pA, nb);
+  if (pl.nlong > 0) {
+    k_il_long_spmv<VW><<<dim3(pl.gxl, pl.gy), blk, 0, st>>>(m, pl.nlong, pl.longs, diag32, alpha, in,
+                                                            (const float*)pl.plong, pA, nb, pl.gxs);
+    note_launch();
+  }
+  k_il_alpha<<<m, 128, 0, st>>>(pA, nb, scal);
+  k_il_update<VW><<<dim3(pl.gxe, pl.gy), blk, 0, st>>>(g->n, m, prec, scal, in, pA, pB, pl.gxe);
+  k_il_beta<<<m, 128, 0, st>>>(pA, pB, pl.gxe, scal, rr_out);
+  k_il_p<VW><<<dim3(pl.gxe, pl.gy), blk, 0, st>>>(g->n, m, prec, scal, in);
+  for (int i = 0; i < 5; ++i) note_launch();
+}
+
+template <int VW>
+static void il_launch_correct(const ILPlan& pl, int32_t n, int m, const double* scal, const float* d, double* x,
+                              cudaStream_t st) {
+  k_il_correct<VW><<<dim3(pl.gxe, pl.gy), dim3(pl.lw, IL_T / pl.lw), 0, st>>>(n, m, scal, d, x);
+  note_launch();
+}
+
+#define IL_DISPATCH(vw, call4, call2, call1) \
+  do {                                       \
+    if ((vw) == 4) call4;                    \
+    else if ((vw) == 2) call2;               \
+    else call1;                              \
+  } while (0)
 
 }  // namespace fcx
 
@@ -1071,13 +1333,14 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   const int32_t n = g->n;
   const int m = n_rhs;
   const double alpha = g->alphas[alpha_idx];
-  const int nb = (n + SV_T - 1) / SV_T;              // blocks of the element-wise kernels
-  const int nbr = (n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK;  // blocks of the row kernels
+  const int nb = (n + SV_T - 1) / SV_T;  // blocks of the element-wise kernels
   const size_t nm = (size_t)n * m;
-  // many right-hand sides: vectors interleaved by column (see k_spmv_pq_il)
-  const bool il = m >= 32;
-  const int gy = (m + 31) / 32;
-  const int gxi = std::max(1, std::min((n + IL_R - 1) / IL_R, 2048 / gy));
+  int coop = 0;
+  FC_CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device));
+  // several right-hand sides: vectors interleaved by column; one: edge tiles
+  // and the inner CG in one cooperative launch
+  const bool il = m >= 2 || !coop;
+  ILPlan il32{}, il64{};  // FP32 products and vectors, FP64 residual
   // scratch: FP64 r64, FP32 r/p/q/d, diag32, partials, scalars
   double* r64 = nullptr;
   float* f32 = nullptr;
@@ -1087,10 +1350,65 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   const size_t nmp = (nm + 3) & ~(size_t)3, np4 = ((size_t)n + 3) & ~(size_t)3;
   FC_CK(cudaMallocAsync((void**)&r64, nm * sizeof(double), st));
   FC_CK(cudaMallocAsync((void**)&f32, (4 * nmp + 2 * np4) * sizeof(float), st));
-  const int npart = std::max(std::max(nb, nbr), il ? gxi : 1);
+  // partial sums per column of the column-major kernels: a few thousand blocks in all
+  const int nbx = std::max(1, std::min(nb, 2048 / m));
+  int npart = nbx;
   double* bi = nullptr;  // interleaved copies of b and x
   double* xi = nullptr;
+  void* seg_mem = nullptr;
+  void* plong = nullptr;
+  const int gy = (m + 31) / 32;  // column tiles of the transposes
   if (il) {
+    // row segments (k_il_seg_count, _fill)
+    const int len = m > 16 ? IL_SEG : IL_SEG_PACK;
+    const size_t n1 = (size_t)n + 1, lmax = (size_t)(g->nnz / len) + 1, smax = (size_t)n + lmax;
+    FC_CK(cudaMallocAsync(&seg_mem, (smax + lmax) * 16 + n1 * 4 * 6, st));
+    int4* segs = (int4*)seg_mem;
+    int4* longs = segs + smax;
+    uint32_t* cnt = (uint32_t*)(longs + lmax);
+    uint32_t *lcnt = cnt + n1, *lrow = cnt + 2 * n1, *off = cnt + 3 * n1, *loff = cnt + 4 * n1, *lidx = cnt + 5 * n1;
+    k_il_seg_count<<<(unsigned)((n1 + 255) / 256), 256, 0, st>>>(n, len, g->rowptr, cnt, lcnt, lrow);
+    FC_LAUNCHED();
+    fc_status ss = exclusive_scan(cnt, off, (int64_t)n1, st);
+    if (ss == FC_OK) ss = exclusive_scan(lcnt, loff, (int64_t)n1, st);
+    if (ss == FC_OK) ss = exclusive_scan(lrow, lidx, (int64_t)n1, st);
+    if (ss != FC_OK) return ss;
+    k_il_seg_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, len, g->rowptr, off, loff, lidx, segs, longs);
+    FC_LAUNCHED();
+    uint32_t h[3];
+    FC_CK(cudaMemcpyAsync(h, off + n, 4, cudaMemcpyDeviceToHost, st));
+    FC_CK(cudaMemcpyAsync(h + 1, loff + n, 4, cudaMemcpyDeviceToHost, st));
+    FC_CK(cudaMemcpyAsync(h + 2, lidx + n, 4, cudaMemcpyDeviceToHost, st));
+    FC_CK(cudaStreamSynchronize(st));
+    FC_CK(cudaMallocAsync(&plong, std::max<size_t>(1, (size_t)h[1] * m * sizeof(double)), st));
+    int nsm = 0;
+    FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
+    auto plan = [&](int vw) {
+      ILPlan p;
+      p.vw = vw;
+      // (two lanes per row leave small graphs with too few warps: n = 5000,
+      // two columns 2.6 ms against 2.3 ms on four lanes; 2^19: 3.7 against 4.5)
+      p.lw = n < (1 << 16) ? 4 : 2;
+      while (p.lw < 32 && p.lw < m) p.lw *= 2;
+      const int rows = IL_T / p.lw;
+      p.gy = (m + p.lw * vw - 1) / (p.lw * vw);
+      const int tot = std::max(1, nsm * 16 / p.gy);  // blocks per column group: about 16 per SM in all
+      p.nseg = (int)h[0];
+      p.nslot = (int)h[1];
+      p.nlong = (int)h[2];
+      p.gxs = std::max(1, std::min((p.nseg + rows - 1) / rows, tot));
+      p.gxl = p.nlong > 0 ? std::max(1, std::min((p.nlong + rows - 1) / rows, tot)) : 0;
+      p.gxe = std::max(1, std::min((n + rows * IL_V - 1) / (rows * IL_V), tot));
+      p.segs = segs;
+      p.longs = longs;
+      p.plong = plong;
+      npart = std::max(npart, std::max(p.gxs + p.gxl, p.gxe));
+      return p;
+    };
+    // values per lane: 16-byte accesses where the columns divide evenly and a
+    // warp's columns are filled
+    il32 = plan(m % 4 == 0 && m >= 128 ? 4 : m % 2 == 0 && m >= 64 ? 2 : 1);
+    il64 = plan(m % 2 == 0 && m >= 64 ? 2 : 1);
     FC_CK(cudaMallocAsync((void**)&bi, nm * sizeof(double), st));
     FC_CK(cudaMallocAsync((void**)&xi, nm * sizeof(double), st));
     const dim3 tg((unsigned)std::min<int64_t>((n + 31) / 32, 1024), (unsigned)std::min<int64_t>(gy, 1024));
@@ -1101,7 +1419,6 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   }
   const double* bv = il ? bi : b;
   double* xv = il ? xi : x;
-  const dim3 gridi(gxi, gy), blki(32, IL_R);
   FC_CK(cudaMallocAsync((void**)&part, (size_t)2 * m * npart * sizeof(double) + 4 * m * sizeof(double), st));
   FC_CK(cudaMallocAsync((void**)&scal, (size_t)8 * m * sizeof(double), st));
   Inner in;
@@ -1118,19 +1435,11 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   const float* prec = jacobi ? inv32 : nullptr;  // z = r * prec
   k_diag32<<<(n + 255) / 256, 256, 0, st>>>(n, g->dw, sigma, alpha, diag32, inv32);
   FC_LAUNCHED();
-  // blocks per column: a few thousand blocks in all, each striding over its
-  // column's chunks (many right-hand sides would otherwise launch millions of
-  // one-chunk blocks); nbx / nbrx partial sums per column
-  const int target = 2048;
-  const int nbx = std::max(1, std::min(nb, target / m));
-  const int nbrx = std::max(1, std::min(nbr, target / m));
-  const dim3 grid(nbx, m);
-  const dim3 gridr(nbrx, m);
   const double inner_tol = 1e-4;
   const int check_every = 8;
   // one right-hand side: row sums by edge tiles (FP64 residual and FP32
   // inner products) and the cooperative inner CG (every CTA resident)
-  const bool tiles = m == 1;
+  const bool tiles = !il;
   const int64_t ntiles = (g->nnz + TL - 1) / TL;
   TileArgs<double> t64{};
   TileArgs<float> t32{};
@@ -1189,33 +1498,27 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     FC_CK(cudaMemcpyAsync(&h_nempty, nempty, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     FC_CK(cudaStreamSynchronize(st));
     fold = h_nempty == 0;
-    int coop = 0, per_sm = 0, nsm = 0;
-    FC_CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device));
+    int per_sm = 0, nsm = 0;
     FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
     tile_grid = (int)std::max<int64_t>(1, std::min<int64_t>((ntiles + TL_W - 1) / TL_W, (int64_t)8 * nsm));
     FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fold ? k_cg1<true> : k_cg1<false>, SV_T, 0));
-    if (coop && per_sm > 0) {
-      cg1_grid = std::min(per_sm, 8) * nsm;
-      FC_CK(cudaMallocAsync((void**)&cg1_part, (3 * (size_t)cg1_grid + 1) * sizeof(double), st));
-    }
+    cg1_grid = std::max(1, std::min(per_sm, 8)) * nsm;
+    FC_CK(cudaMallocAsync((void**)&cg1_part, (3 * (size_t)cg1_grid + 1) * sizeof(double), st));
   }
   std::vector<double> h_rr(m), h_bb(m), h_scal((size_t)8 * m, 0.0), h_in(m);
   int used = 0;
   fc_status result = FC_ENOCONV;
   for (int outer = 0; outer < 64; ++outer) {
-    int nres = il ? gxi : nbrx;  // residual partials per column
+    const int nres = il ? il64.gxs + il64.gxl : nbx;  // residual partials per column
     if (il) {
-      k_resid64_il<<<gridi, blki, 0, st>>>(n, m, g->rowptr, g->colidx, g->w, g->dw, sigma, alpha, bv, xv, r64, pA, pB,
-                                           gxi);
-    } else if (tiles) {
+      if (il64.vw == 2) il_launch_resid<2>(il64, g, m, sigma, alpha, bv, xv, r64, pA, pB, st);
+      else il_launch_resid<1>(il64, g, m, sigma, alpha, bv, xv, r64, pA, pB, st);
+    } else {
       if (ntiles > 0) {
         k_tile_rowsum64<<<tile_grid, SV_T, 0, st>>>(t64, x, ntiles);
         FC_LAUNCHED();
       }
       k_resid_rows<<<nbx, SV_T, 0, st>>>(n, t64, g->dw, sigma, alpha, b, x, r64, pA, pB);
-      nres = nbx;
-    } else {
-      k_resid64<<<gridr, SV_T, 0, st>>>(n, g->rowptr, g->colidx, g->w, g->dw, sigma, alpha, b, x, r64, pA, pB, nbrx);
     }
     FC_LAUNCHED();
     k_colsum<<<m, SV_T, 0, st>>>(pA, nres, sums);
@@ -1223,7 +1526,14 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     k_colsum<<<m, SV_T, 0, st>>>(pB, nres, sums + m);
     fcx::note_launch();
     if (sigma == 0.0) {  // singular L: keep the residual in L's range
-      k_proj_mean<<<m, SV_T, 0, st>>>(n, m, il, r64, sums);
+      const int64_t sv = il ? m : 1, sj = il ? 1 : n;
+      k_col_part<<<dim3(nbx, m), SV_T, 0, st>>>(n, r64, sv, sj, pA, nbx);
+      FC_LAUNCHED();
+      k_colsum<<<m, SV_T, 0, st>>>(pA, nbx, sums);
+      FC_LAUNCHED();
+      k_col_shift<<<dim3(nbx, m), SV_T, 0, st>>>(n, r64, sv, sj, sums, r64, pB, nbx);
+      FC_LAUNCHED();
+      k_colsum<<<m, SV_T, 0, st>>>(pB, nbx, sums);
       FC_LAUNCHED();
     }
     FC_CK(cudaMemcpyAsync(h_rr.data(), sums, m * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1244,13 +1554,15 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     if (used >= max_iter) break;
     FC_CK(cudaMemcpyAsync(scal, h_scal.data(), (size_t)8 * m * sizeof(double), cudaMemcpyHostToDevice, st));
     if (il)
-      k_inner_init_il<<<gridi, blki, 0, st>>>(n, m, r64, prec, scal, in, pA, pB, gxi);
+      IL_DISPATCH(il32.vw, il_launch_init<4>(il32, n, m, r64, prec, scal, in, pA, pB, st),
+                  il_launch_init<2>(il32, n, m, r64, prec, scal, in, pA, pB, st),
+                  il_launch_init<1>(il32, n, m, r64, prec, scal, in, pA, pB, st));
     else
-      k_inner_init<<<grid, SV_T, 0, st>>>(n, r64, prec, scal, in, pA, pB, nbx);
+      k_inner_init<<<nbx, SV_T, 0, st>>>(n, r64, prec, scal, in, pA, pB, nbx);
     FC_LAUNCHED();
-    k_colsum<<<m, SV_T, 0, st>>>(pA, il ? gxi : nbx, sums);
+    k_colsum<<<m, SV_T, 0, st>>>(pA, il ? il32.gxe : nbx, sums);
     fcx::note_launch();
-    k_colsum<<<m, SV_T, 0, st>>>(pB, il ? gxi : nbx, sums + m);
+    k_colsum<<<m, SV_T, 0, st>>>(pB, il ? il32.gxe : nbx, sums + m);
     fcx::note_launch();
     FC_CK(cudaMemcpyAsync(h_in.data(), sums, m * sizeof(double), cudaMemcpyDeviceToHost, st));
     FC_CK(cudaMemcpyAsync(h_rr.data(), sums + m, m * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1284,35 +1596,11 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
       used += done;
     }
     int it = 0;
-    while (cg1_grid == 0 && used < max_iter) {
-      if (il)
-        k_spmv_pq_il<<<gridi, blki, 0, st>>>(n, m, g->rowptr, g->colidx, g->w, diag32, (float)alpha, in, pA, gxi);
-      else
-        k_spmv_pq<<<gridr, SV_T, 0, st>>>(n, g->rowptr, g->colidx, g->w, diag32, (float)alpha, in, pA, nbrx);
-      FC_LAUNCHED();
-      // pq -> scal[j*8+1]
-      k_colsum<<<m, SV_T, 0, st>>>(pA, il ? gxi : nbrx, sums);
-      fcx::note_launch();
-      k_put_scal<<<(m + 127) / 128, 128, 0, st>>>(m, sums, 1, 1, scal);
-      FC_LAUNCHED();
-      if (il)
-        k_inner_update_il<<<gridi, blki, 0, st>>>(n, m, prec, scal, in, pA, pB, gxi);
-      else
-        k_inner_update<<<grid, SV_T, 0, st>>>(n, prec, scal, in, pA, pB, nbx);
-      FC_LAUNCHED();
-      k_colsum<<<m, SV_T, 0, st>>>(pA, il ? gxi : nbx, sums);
-      fcx::note_launch();
-      k_colsum<<<m, SV_T, 0, st>>>(pB, il ? gxi : nbx, sums + m);
-      fcx::note_launch();
-      k_put_scal<<<(m + 127) / 128, 128, 0, st>>>(m, sums, 2, 2, scal);  // scal[2] <- sums[0..m), scal[3] <- sums[m..2m)
-      FC_LAUNCHED();
-      if (il)
-        k_inner_p_il<<<gridi, blki, 0, st>>>(n, m, prec, scal, in);
-      else
-        k_inner_p<<<grid, SV_T, 0, st>>>(n, prec, scal, in);
-      FC_LAUNCHED();
-      k_scal_shift<<<(m + 127) / 128, 128, 0, st>>>(m, scal);
-      fcx::note_launch();
+    while (il && used < max_iter) {
+      IL_DISPATCH(il32.vw, il_launch_iter<4>(il32, g, m, prec, diag32, (float)alpha, scal, in, pA, pB, sums + m, st),
+                  il_launch_iter<2>(il32, g, m, prec, diag32, (float)alpha, scal, in, pA, pB, sums + m, st),
+                  il_launch_iter<1>(il32, g, m, prec, diag32, (float)alpha, scal, in, pA, pB, sums + m, st));
+      FC_CK(cudaGetLastError());
       ++used;
       ++it;
       if (it == 1 || it == 2 || it == 4 || it % check_every == 0) {
@@ -1325,9 +1613,11 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
       }
     }
     if (il)
-      k_correct_il<<<gridi, blki, 0, st>>>(n, m, scal, in.d, xv);
+      IL_DISPATCH(il32.vw, il_launch_correct<4>(il32, n, m, scal, in.d, xv, st),
+                  il_launch_correct<2>(il32, n, m, scal, in.d, xv, st),
+                  il_launch_correct<1>(il32, n, m, scal, in.d, xv, st));
     else
-      k_correct<<<grid, SV_T, 0, st>>>(n, scal, in.d, x);
+      k_correct<<<nbx, SV_T, 0, st>>>(n, scal, in.d, x);
     FC_LAUNCHED();
   }
   if (il) {
@@ -1336,6 +1626,8 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     FC_LAUNCHED();
     FC_CK(cudaFreeAsync(bi, st));
     FC_CK(cudaFreeAsync(xi, st));
+    FC_CK(cudaFreeAsync(seg_mem, st));
+    FC_CK(cudaFreeAsync(plong, st));
   }
   FC_CK(cudaFreeAsync(r64, st));
   FC_CK(cudaFreeAsync(f32, st));
@@ -1390,21 +1682,17 @@ extern "C" fc_status fc_pivot_solve(fc_graph* g, int32_t alpha_idx, double* x, d
   return s;
 }
 
-// Column sums of an [m][n] block (one block per column, fixed order) and the
-// mean of each column subtracted: out[j][v] = in[j][v] - sum_j / n.
-__global__ void k_col_mean_sub(int32_t n, const double* __restrict__ in, double* __restrict__ out) {
-  __shared__ double red[SV_T];
-  const size_t off = (size_t)blockIdx.x * n;
-  double s = 0.0;
-  for (int64_t v = threadIdx.x; v < n; v += SV_T) s += in[off + v];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = SV_T / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  const double mean = red[0] / (double)n;
-  for (int64_t v = threadIdx.x; v < n; v += SV_T) out[off + v] = in[off + v] - mean;
+// out[j][v] = in[j][v] - mean_j for the columns of an [m][n] block (in place
+// when out is in); part: [m][nb + 1] scratch
+static fc_status sub_col_means(int32_t n, int m, const double* in, double* out, double* part, int nb, cudaStream_t st) {
+  double* sums = part + (size_t)m * nb;
+  k_col_part<<<dim3(nb, m), SV_T, 0, st>>>(n, in, 1, n, part, nb);
+  FC_LAUNCHED();
+  k_colsum<<<m, SV_T, 0, st>>>(part, nb, sums);
+  FC_LAUNCHED();
+  k_col_shift<<<dim3(nb, m), SV_T, 0, st>>>(n, in, 1, n, sums, out, nullptr, nb);
+  FC_LAUNCHED();
+  return FC_OK;
 }
 
 extern "C" fc_status fc_laplacian_solve(fc_graph* g, const double* b, double* x, int32_t n_rhs, double rel_tol,
@@ -1420,16 +1708,20 @@ extern "C" fc_status fc_laplacian_solve(fc_graph* g, const double* b, double* x,
   cudaStream_t st = (cudaStream_t)stream;
   const int32_t n = g->n;
   double* rhs = nullptr;
+  double* part = nullptr;
+  const int nb = std::max(1, std::min((n + SV_T - 1) / SV_T, 2048 / n_rhs));
   FC_CK(cudaMallocAsync((void**)&rhs, (size_t)n * n_rhs * sizeof(double), st));
+  FC_CK(cudaMallocAsync((void**)&part, (size_t)n_rhs * (nb + 1) * sizeof(double), st));
   // b projected onto the range of L (the complement of span(1))
-  k_col_mean_sub<<<n_rhs, SV_T, 0, st>>>(n, b, rhs);
-  FC_LAUNCHED();
+  const fc_status sb = sub_col_means(n, n_rhs, b, rhs, part, nb, st);
+  if (sb != FC_OK) return sb;
   const fc_status s = solve_impl(g, 0, rhs, x, n_rhs, rel_tol, max_iter, iters_out, st, true, 0.0);
   if (s == FC_OK || s == FC_ENOCONV) {
     // the mean-zero solution: L^+ b
-    k_col_mean_sub<<<n_rhs, SV_T, 0, st>>>(n, x, x);
-    FC_LAUNCHED();
+    const fc_status sx = sub_col_means(n, n_rhs, x, x, part, nb, st);
+    if (sx != FC_OK) return sx;
   }
+  FC_CK(cudaFreeAsync(part, st));
   FC_CK(cudaFreeAsync(rhs, st));
   FC_CK(cudaStreamSynchronize(st));
   return s;
