@@ -136,7 +136,7 @@ __global__ void k_p_root(int32_t n, const uint4* __restrict__ rinfo, double* __r
 // block (k_ts_sort).  Larger k: stable LSD radix sort of all pairs (inputs in id
 // order, so equal keys keep ascending ids).  Bound by launches and passes over
 // diag: measured on GB300 for k = 10 against the sort, whole calls: n = 1000 270 ->
-// 53 us, n = 2^20 371 -> 63 us, n = 2^22 (65 distinct values) 580 -> 309 us.
+// 53 us, n = 2^20 371 -> 63 us, n = 2^22 (R-MAT) 580 -> 309 us.
 // ---------------------------------------------------------------------------
 constexpr int TK_TILE = 1024;
 
@@ -209,7 +209,7 @@ __global__ void k_tk_scatter(int32_t n, const uint64_t* __restrict__ kin, const 
 constexpr int TS_T = 512;
 constexpr int TS_BITS = 11;
 constexpr int TS_BINS = 1 << TS_BITS;
-constexpr int TS_PASSES = 9;   // key digits 11 x 5 + 9, id digits 11 + 11 + 8 (ids below 2^30)
+constexpr int TS_PASSES = 9;   // key digits 11 x 5 + 9, id digits 11 + 11 + 9 (31 bits: every id)
 constexpr int TS_CAP = 1024;   // pairs on the prefix that end the selection
 constexpr int TS_N = 4096;     // pairs sorted by one block
 constexpr int TS_K = TS_N - TS_CAP;
@@ -220,8 +220,8 @@ struct TSPrefix {
   uint64_t key;  // digits of the key so far, in place
   uint32_t id;
 };
-__device__ __forceinline__ int ts_shift(int p) { return p < 5 ? 53 - 11 * p : p == 5 ? 0 : p == 6 ? 19 : p == 7 ? 8 : 0; }
-__device__ __forceinline__ int ts_bits(int p) { return p == 5 ? 9 : p == 8 ? 8 : TS_BITS; }
+__device__ __forceinline__ int ts_shift(int p) { return p < 5 ? 53 - 11 * p : p == 5 ? 0 : p == 6 ? 20 : p == 7 ? 9 : 0; }
+__device__ __forceinline__ int ts_bits(int p) { return p == 5 || p == 8 ? 9 : TS_BITS; }
 __device__ __forceinline__ uint32_t ts_digit(uint64_t key, uint32_t id, int p) {
   const uint64_t x = p < 6 ? key : (uint64_t)id;
   return (uint32_t)(x >> ts_shift(p)) & ((1u << ts_bits(p)) - 1u);
