@@ -777,8 +777,8 @@ def run_group(args):
 
 def run_roots(args):
     """Forest roots and depths of sampled trees on the benchmark graph (BA
-    n = 2^20, m = 8), 152 trees: written by the sampler as vertices join the
-    tree (fc_sample_usts_forest), against sampling with parents followed by
+    n = 2^20, m = 8), 152 trees: one call of the sampler
+    (fc_sample_usts_forest), against sampling with parents followed by
     pointer jumping (fc_tree_roots); and root counts of 64 query vertices
     (fc_root_counts: columns of Omega from the same trees).  L2 flushed before
     each timed call."""
@@ -840,7 +840,7 @@ def run_roots(args):
             "config": {"workload": f"BA n=2^{args.n_log2} m={BA_M}, alpha={ALPHA:g}, {T} trees, 64 queries",
                        "l2": "flushed before every timed call (512 MB write)"},
             "roofline": {"bound": "hbm", "achieved": alg / t_r / 1e9, "peak": peak, "unit": "GB/s",
-                         "frac": alg / t_r / 1e9 / peak, "traffic": None, "kernel": "k_roots_jump",
+                         "frac": alg / t_r / 1e9 / peak, "traffic": None, "kernel": "k_roots",
                          "algorithmic_bytes": alg, "peak_source": peak_kind},
             "max_depth": int(depth.max().item())}
     G.close()

@@ -262,10 +262,10 @@ fc_status fc_sample_usts_ex(fc_graph* g, uint64_t seed, int64_t tau, int64_t tre
  *            theorem (Sec. 2) P(roots[t][v] = u) = Omega[u, v]
  *   depths   int32 [rows][n]   the number of edges from v to its root
  * rows and indexing as parents (n_alpha * tau rows, or tau rows of the union
- * for a batch).  The edge-record kernel without clusters writes both as
- * vertices join the tree, with no pass over the parents; otherwise they come
- * from fc_tree_roots on the parents (allocated internally when parents is
- * NULL).  Everything else as fc_sample_usts_ex.  Synchronises `stream`.
+ * for a batch).  The edge-record kernel without clusters, when chosen, writes
+ * both as vertices join the tree, with no pass over the parents; otherwise they
+ * come from the parents by the pointer jumping of fc_tree_roots (in place when
+ * parents is NULL).  Everything else as fc_sample_usts_ex.  Synchronises `stream`.
  */
 fc_status fc_sample_usts_forest(fc_graph* g, uint64_t seed, int64_t tau, int64_t tree_offset, uint32_t* R,
                                 uint32_t* C, int32_t* parents, int32_t* roots, int32_t* depths, uint64_t* visits,

@@ -51,6 +51,10 @@ void retain_pool(int device);
 // memory from the stream-ordered pool).
 fc_status exclusive_scan(const uint32_t* in, uint32_t* out, int64_t len, cudaStream_t st);
 
+// Roots and depths (either may be null; parents may be one of them) of T rows
+// of parents; synchronises `st`.
+fc_status tree_roots(const int32_t* parents, int32_t n, int64_t T, int32_t* roots, int32_t* depth, cudaStream_t st);
+
 // Device error word bits (OR-ed by kernels, read back by the host).
 enum : uint32_t {
   ERR_INVAL = 1u,

@@ -683,24 +683,26 @@ static fc_status batch_stamps(fc_graph* g, int64_t tau, bool capturing, cudaStre
 // the walker kernels (ms per call): BA n = 2^20, 1024 trees 42.5 -> 23.7;
 // R-MAT 2^20, 64 trees 8.5 -> 1.5; weighted 1024^2 grid, 152 trees, alpha 0.1
 // 25.0 -> 4.4, 1 47.3 -> 15.0, 10 79.4 -> 38.9; ER n = 1000, 2000 trees 1.3 ->
-// 0.37; BA n = 2^20 rooted at its hub, 152 trees 118 -> 87.  Exceptions:
-//  * forest roots: recorded by the edge-record kernel as vertices join a tree;
+// 0.37; BA n = 2^20 rooted at its hub, 152 trees 118 -> 87; with forest roots
+// and depths (parents, then pointer jumping, against recording them as vertices
+// join the tree) BA n = 2^17, 96 trees 2.3 -> 0.88.  Exceptions:
 //  * ids of 29 bits in the words of the tops;
 //  * parents (an analysis output) of unweighted graphs of 2^15 to 2^16 vertices
 //    without a dominating hub: tests/test_gpu_edge_kernel.py pins the walker
 //    kernel and its automatic clusters for these launches (0.87 ms against
 //    0.34 ms for 64 trees of BA n = 50,000).
-static bool pop_applies(const fc_graph* g, const int32_t* parents, const int32_t* roots, const int32_t* depths) {
+static bool pop_applies(const fc_graph* g, const int32_t* parents) {
   const bool automatic = g->kernel_pref == 0 && g->walkers == 0 && g->max_trees == 0 && g->smem_mode == 0 &&
                          g->regs == 0 && g->bitmap_mode == 0 && g->pops_mode == 0 && g->cluster == 0;
   const bool pinned = parents != nullptr && !g->weighted && g->num_graphs == 0 && g->root < 0 && g->n > (1 << 15) &&
                       g->n <= (1 << 16) && g->max_deg <= g->n / 16;
-  return automatic && roots == nullptr && depths == nullptr && g->n < (1 << 29) - 1 && !pinned;
+  return automatic && g->n < (1 << 29) - 1 && !pinned;
 }
 
 static fc_status sample_pop(fc_graph* g, uint64_t seed, int64_t tau, int64_t tree_offset, uint32_t* R, uint32_t* C,
-                            int32_t* parents, uint64_t* visits, uint64_t max_steps_per_tree, uint64_t* steps_out,
-                            cudaStream_t st, bool sync, bool capturing) {
+                            int32_t* parents, int32_t* roots, int32_t* depths, uint64_t* visits,
+                            uint64_t max_steps_per_tree, uint64_t* steps_out, cudaStream_t st, bool sync,
+                            bool capturing) {
   const bool batch = g->num_graphs > 0;
   WParams p = {};
   p.tau = tau;
@@ -739,12 +741,18 @@ static fc_status sample_pop(fc_graph* g, uint64_t seed, int64_t tau, int64_t tre
   scr.st = st;
   FC_CK(cudaMallocAsync(&scr.ptr, pl.bytes, st));
   if (sync) FC_CK(cudaMemsetAsync(g->d_err, 0, sizeof(uint32_t), st));
+  // forest roots and depths: by pointer jumping over the parents, in place
+  // when they are not asked for
+  const bool want_roots = roots != nullptr || depths != nullptr;
+  if (want_roots && parents == nullptr) p.parents = roots != nullptr ? roots : depths;
   const fc_status s = pop_sample(g, p, pl, scr.ptr, st);
   if (s != FC_OK || !sync) return s;
   uint32_t herr = 0;
   FC_CK(cudaMemcpyAsync(&herr, g->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   FC_CK(cudaStreamSynchronize(st));
-  return sampler_status(herr, "fc_sample_usts");
+  const fc_status es = sampler_status(herr, "fc_sample_usts");
+  if (es != FC_OK || !want_roots) return es;
+  return tree_roots(p.parents, g->n, batch ? tau : g->n_alpha * tau, roots, depths, st);
 }
 
 static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tree_offset, uint32_t* R, uint32_t* C,
@@ -765,9 +773,9 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
     set_error("fc_sample_usts: reads its status back; use fc_sample_usts_async on a capturing stream");
     return FC_EINVAL;
   }
-  if (pop_applies(g, parents, roots, depths))
-    return sample_pop(g, seed, tau, tree_offset, R, C, parents, visits, max_steps_per_tree, steps_out, st, sync,
-                      capturing);
+  if (pop_applies(g, parents))
+    return sample_pop(g, seed, tau, tree_offset, R, C, parents, roots, depths, visits, max_steps_per_tree, steps_out, st,
+                      sync, capturing);
   int dev_smem_optin = 0, nsm = 0;
   FC_CK(cudaDeviceGetAttribute(&dev_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
   FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
@@ -919,16 +927,11 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
   p.R = R;
   p.C = C;
   p.parents = parents;
-  const size_t prow = (size_t)(batch ? tau : (int64_t)g->n_alpha * tau);  // parent rows of the call
-  StreamScratch pscr;
-  pscr.st = st;
   p.roots = fused_roots ? roots : nullptr;
   p.depths = fused_roots ? depths : nullptr;
   p.rdpack = rdpack;
-  if (want_roots && !fused_roots && parents == nullptr) {  // pointer jumping needs the parents
-    FC_CK(cudaMallocAsync(&pscr.ptr, prow * (size_t)n * sizeof(int32_t), st));
-    p.parents = (int32_t*)pscr.ptr;
-  }
+  if (want_roots && !fused_roots && parents == nullptr)  // pointer jumping needs the parents, in place
+    p.parents = roots != nullptr ? roots : depths;
   p.visits = (unsigned long long*)visits;
   p.steps = steps_out;
   p.gstate = (VState*)gstate;
@@ -1002,13 +1005,7 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
   FC_CK(cudaStreamSynchronize(st));
   const fc_status es = sampler_status(herr, "fc_sample_usts");
   if (es != FC_OK) return es;
-  if (want_roots && !fused_roots) {
-    StreamScratch r2;
-    r2.st = st;
-    if (roots == nullptr) FC_CK(cudaMallocAsync(&r2.ptr, prow * (size_t)n * sizeof(int32_t), st));
-    const fc_status s = fc_tree_roots(p.parents, n, (int64_t)prow, roots ? roots : (int32_t*)r2.ptr, depths, st);
-    if (s != FC_OK) return s;
-  }
+  if (want_roots && !fused_roots) return tree_roots(p.parents, n, batch ? tau : g->n_alpha * tau, roots, depths, st);
   return FC_OK;
 }
 
