@@ -13,7 +13,13 @@
 // W1[128][4], b1[128], w2[128], b2.  Every kernel reads them rounded to BF16
 // (round to nearest even) and accumulates in FP32.  The hidden layer has K = 4
 // and the output layer N = 1, so these are per-vertex dot products on the
-// CUDA cores, bound by reading the 16-byte feature rows.
+// CUDA cores, bound by issue slots: 5 FMAs, a maximum and the weights' loads per
+// vertex and hidden unit, against a 16-byte feature row per vertex.  So a thread
+// of the forward pass takes eight vertices per load of a unit's weights, and a
+// lane of the gradient pass four units per load of a vertex's features.
+// Measured on GB300 (whole calls, against one vertex and one unit): forward pass
+// n = 2^22 190 -> 139 us; loss and gradient n = 2^22 475 -> 397, 2^18 53 -> 42.
+// Packed FP32 pairs (fma.rn.f32x2) issued as many instructions: 200 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -31,71 +37,108 @@ constexpr int MLP_T = 128;          // threads per block (one hidden unit each i
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-__device__ __forceinline__ double p_of(const uint4& ri) {
+// p = T 2^-53 rounded to FP32.  T <= 2^53, so this is the FP64 value rounded
+// once (the FP64 pipe would be the cost: two results per clock and SM).
+__device__ __forceinline__ float p_of(const uint4& ri) {
   const uint64_t T = (uint64_t)ri.z | ((uint64_t)ri.w << 32);
-  return (double)T * 0x1.0p-53;
+  return __ull2float_rn(T) * 0x1.0p-53f;
 }
 
 // Sum over neighbours of their degree, s2[v] = sum over w in N(v) of deg(w).
-// A warp takes chunks of NDS_CHUNK consecutive CSR entries and walks each in
-// steps of 32: lane i reads entry e0 + i (coalesced column indices), finds its
-// row among the 32 row ends that follow the step's first row (a binary search
-// over the warp's registers; an entry beyond them, after empty rows, searches
-// the row pointers itself), and the lanes of one row add their neighbours'
-// degrees with a segmented warp sum whose last lane adds the total to s2 (one
-// atomic per row segment, so a hub row is shared by many warps).  The totals
-// are integers: any order of the additions gives the same result.
-constexpr int NDS_CHUNK = 32 * 32;
+// A block takes consecutive tiles of NDS_TILE CSR entries whatever rows they
+// belong to: every thread has NDS_U neighbour gathers in flight, the tile's
+// prefix sums go to shared memory, and a thread per row of the tile takes the
+// difference over its entries.  Rows inside the tile are stored, rows that
+// cross tiles add their parts (integers: any order gives the same result).
+// The gathers of the next tile and the column indices of the one after it are
+// under way meanwhile; the first tile's first row comes from a 32-way search,
+// the later ones' from the tile before.  Bound by the gathers of deg.  (Before:
+// a warp walked 1024 entries in 32 dependent steps.  Features on GB300, whole
+// calls: R-MAT n = 2^16 37 -> 25 us, 2^18 64 -> 49, 2^22 786 -> 606.)
+constexpr int NDS_T = 256;
+constexpr int NDS_U = 8;
+constexpr int NDS_TILE = NDS_T * NDS_U;
 constexpr unsigned NDS_FULL = 0xffffffffu;
-__device__ __forceinline__ int32_t row_of_entry(const int64_t* __restrict__ rowptr, int32_t lo, int32_t hi,
-                                                int64_t e) {
-  // the row v in [lo, hi] with rowptr[v] <= e < rowptr[v + 1] (the last such v: rows may be empty)
-  while (lo < hi) {
-    const int32_t mid = lo + (hi - lo + 1) / 2;
-    if (rowptr[mid] <= e) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
+__device__ __forceinline__ int nds_pad(int i) { return i + (i >> 3); }  // eight per thread without bank conflicts
 
-__global__ void k_nbr_deg_sum(int32_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
-                              const int32_t* __restrict__ colidx, const int32_t* __restrict__ deg,
-                              unsigned long long* __restrict__ s2) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t c0 = warp * NDS_CHUNK; c0 < nnz; c0 += nwarps * NDS_CHUNK) {
-    const int64_t c1 = c0 + NDS_CHUNK < nnz ? c0 + NDS_CHUNK : nnz;
-    int32_t r = row_of_entry(rowptr, 0, n - 1, c0);  // row of the step's first entry (warp-uniform)
-    for (int64_t e0 = c0; e0 < c1; e0 += 32) {
-      const int64_t e = e0 + lane;
-      const bool ok = e < c1;
-      unsigned long long val = ok ? (unsigned long long)deg[colidx[e]] : 0ull;
-      // end of row r + k in lane k; the count of ends <= e is the lane's row offset
-      const int32_t rk = r + 1 + lane;
-      const int64_t endk = rk <= n ? rowptr[rk] : INT64_MAX;
-      int32_t row = r;
-      if (__shfl_sync(NDS_FULL, endk, 0) <= e0 + 31) {  // the step crosses a row end
-        int32_t cnt = 0;
+__global__ void __launch_bounds__(NDS_T, 6) k_nbr_deg_sum(int32_t n, int64_t nnz, const int64_t* __restrict__ rowptr,
+                                                          const int32_t* __restrict__ colidx,
+                                                          const int32_t* __restrict__ deg, int64_t per,
+                                                          unsigned long long* __restrict__ s2) {
+  __shared__ unsigned long long P[NDS_TILE + NDS_TILE / 8 + 1];  // exclusive prefix sums, padded
+  __shared__ __align__(16) uint32_t val[NDS_TILE];
+  __shared__ unsigned long long wsum[NDS_T / 32];
+  __shared__ int32_t first[2];  // first row of the tile, by the tile's parity
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t b0 = (int64_t)blockIdx.x * per * NDS_TILE;
+  const int64_t b1 = b0 + per * NDS_TILE < nnz ? b0 + per * NDS_TILE : nnz;  // this block's entries
+  int32_t c[NDS_U];
+  uint32_t d[NDS_U];
+  auto cols = [&](int64_t e0) {
 #pragma unroll
-        for (int b = 16; b >= 1; b >>= 1) {
-          const int64_t probe = __shfl_sync(NDS_FULL, endk, cnt + b - 1);
-          if (probe <= e) cnt += b;
-        }
-        if (__shfl_sync(NDS_FULL, endk, cnt) <= e) ++cnt;
-        row = cnt < 32 ? r + cnt : row_of_entry(rowptr, r + 32, n - 1, e);
-      }
-      // segmented inclusive sum over lanes of the same row (rows do not decrease with the lane)
+    for (int k = 0; k < NDS_U; ++k) {
+      const int64_t e = e0 + k * NDS_T + threadIdx.x;
+      c[k] = e < b1 ? __ldcs(colidx + e) : -1;
+    }
+  };
+  auto gather = [&]() {
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const unsigned long long ov = __shfl_up_sync(NDS_FULL, val, d);
-        const int32_t orow = __shfl_up_sync(NDS_FULL, row, d);
-        if (lane >= d && orow == row) val += ov;
-      }
-      const int32_t nrow = __shfl_down_sync(NDS_FULL, row, 1);
-      const bool nok = __shfl_down_sync(NDS_FULL, ok ? 1 : 0, 1) != 0;
-      if (ok && val != 0ull && (lane == 31 || !nok || nrow != row)) atomicAdd(&s2[row], val);
-      r = __shfl_sync(NDS_FULL, row, 31);
+    for (int k = 0; k < NDS_U; ++k) d[k] = c[k] >= 0 ? (uint32_t)__ldg(deg + c[k]) : 0u;
+  };
+  cols(b0);
+  gather();
+  cols(b0 + NDS_TILE);
+  if (wid == 0) {  // the last row v with rowptr[v] <= b0: rowptr[lo] <= b0 < rowptr[hi]
+    int32_t lo = 0, hi = n;
+    while (hi - lo > 1) {
+      const int32_t step = hi - lo >= 64 ? (hi - lo) / 32 : 1;
+      const int64_t x = (int64_t)lo + (int64_t)step * (lane + 1);
+      const int cnt = __popc(__ballot_sync(NDS_FULL, x < hi && rowptr[x < hi ? x : lo] <= b0));
+      lo += step * cnt;
+      if (cnt < 32 && hi - lo > step) hi = lo + step;
+    }
+    if (lane == 0) first[0] = lo;
+  }
+  int par = 0;
+  for (int64_t e0 = b0; e0 < b1; e0 += NDS_TILE, par ^= 1) {
+    const int64_t e1 = e0 + NDS_TILE < b1 ? e0 + NDS_TILE : b1;
+#pragma unroll
+    for (int k = 0; k < NDS_U; ++k) val[k * NDS_T + threadIdx.x] = d[k];
+    gather();
+    cols(e0 + 2 * NDS_TILE);
+    __syncthreads();
+    unsigned long long x[NDS_U], s = 0;
+    const uint4* v4 = reinterpret_cast<const uint4*>(val + threadIdx.x * NDS_U);
+    const uint4 va = v4[0], vb = v4[1];
+    const uint32_t v[NDS_U] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
+#pragma unroll
+    for (int k = 0; k < NDS_U; ++k) {
+      x[k] = s;
+      s += v[k];
+    }
+    unsigned long long inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(NDS_FULL, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[wid] = inc;
+    __syncthreads();
+    unsigned long long base = inc - s;
+    for (int q = 0; q < wid; ++q) base += wsum[q];
+#pragma unroll
+    for (int k = 0; k < NDS_U; ++k) P[nds_pad(threadIdx.x * NDS_U + k)] = base + x[k];
+    if (threadIdx.x == NDS_T - 1) P[nds_pad(NDS_TILE)] = base + s;
+    __syncthreads();
+    for (int64_t r = first[par] + (int64_t)threadIdx.x; r < n; r += NDS_T) {
+      const int64_t r0 = rowptr[r], r1 = rowptr[r + 1];
+      if (r0 >= e1) break;
+      if (r1 >= e1) first[par ^ 1] = (int32_t)r;  // one row: the last that starts before e1
+      const int64_t a0 = r0 > e0 ? r0 : e0, a1 = r1 < e1 ? r1 : e1;
+      if (a1 <= a0) continue;  // an empty row (zero already), or one that ended with the tile before
+      const unsigned long long sum = P[nds_pad((int)(a1 - e0))] - P[nds_pad((int)(a0 - e0))];
+      if (a0 == r0 && a1 == r1) s2[r] = sum;
+      else atomicAdd(&s2[r], sum);
     }
   }
 }
@@ -112,108 +155,207 @@ __global__ void k_features(int32_t n, double alpha_s, const double* __restrict__
   }
 }
 
-__device__ __forceinline__ void load_params(const float* __restrict__ params, float* sw) {
-  for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) sw[i] = bf16r(params[i]);
+// The (BF16-valued) weights of a hidden unit: two loads
+struct __align__(16) Unit {
+  float4 w;      // W1[j]
+  float b, w2;   // b1[j], w2[j]
+  float pad[2];
+};
+__device__ __forceinline__ void load_params(const float* __restrict__ params, Unit* su) {
+  for (int j = threadIdx.x; j < HID; j += blockDim.x) {
+    const float* w = params + OFF_W1 + j * NF;
+    su[j].w = make_float4(bf16r(w[0]), bf16r(w[1]), bf16r(w[2]), bf16r(w[3]));
+    su[j].b = bf16r(params[OFF_B1 + j]);
+    su[j].w2 = bf16r(params[OFF_W2 + j]);
+  }
   __syncthreads();
 }
 
-// z = w2 . relu(W1 x + b1) + b2 with the (BF16-valued) weights in shared memory
-__device__ __forceinline__ float mlp_z(const float* sw, const float4& x) {
-  float z = sw[OFF_B2];
-#pragma unroll 8
-  for (int j = 0; j < HID; ++j) {
-    const float4 w = *reinterpret_cast<const float4*>(sw + OFF_W1 + j * NF);  // one 16-byte load
-    float pre = sw[OFF_B1 + j];
-    pre = fmaf(w.x, x.x, pre);
-    pre = fmaf(w.y, x.y, pre);
-    pre = fmaf(w.z, x.z, pre);
-    pre = fmaf(w.w, x.w, pre);
-    z = fmaf(sw[OFF_W2 + j], fmaxf(pre, 0.0f), z);
-  }
-  return z;
+// W1[j] x + b1[j]
+__device__ __forceinline__ float mlp_pre(const float4& w, float b, const float4& x) {
+  float pre = fmaf(w.x, x.x, b);
+  pre = fmaf(w.y, x.y, pre);
+  pre = fmaf(w.z, x.z, pre);
+  return fmaf(w.w, x.w, pre);
 }
 
+// z = w2 . relu(W1 x + b1) + b2 of NV vertices
+template <int NV>
+__device__ __forceinline__ void mlp_z(const Unit* su, float b2, const float4 (&x)[NV], float (&z)[NV]) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) z[i] = b2;
+#pragma unroll 4
+  for (int j = 0; j < HID; ++j) {
+    const float4 w = su[j].w;
+    const float2 u = *reinterpret_cast<const float2*>(&su[j].b);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) z[i] = fmaf(u.y, fmaxf(mlp_pre(w, u.x, x[i]), 0.0f), z[i]);
+  }
+}
+
+__device__ __forceinline__ float mlp_g(float z, const uint4& ri) {
+  const float s = 1.0f / (1.0f + expf(-z));
+  const float p = p_of(ri);
+  return p + (1.0f - p) * s;
+}
+
+constexpr int MLP_NV = 8;  // vertices per thread of the forward pass
 __global__ void __launch_bounds__(MLP_T) k_mlp_forward(int32_t n, const float4* __restrict__ X,
                                                        const uint4* __restrict__ rinfo,
                                                        const float* __restrict__ params, float* __restrict__ gout) {
-  __shared__ __align__(16) float sw[NPARAM];
-  load_params(params, sw);
-  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const float z = mlp_z(sw, X[v]);
-    const float s = 1.0f / (1.0f + expf(-z));
-    const float p = (float)p_of(rinfo[v]);
-    gout[v] = p + (1.0f - p) * s;
+  __shared__ Unit su[HID];
+  load_params(params, su);
+  const float b2 = bf16r(params[OFF_B2]);
+  const int64_t step = MLP_NV * MLP_T;
+  for (int64_t base = blockIdx.x * step; base < n; base += gridDim.x * step) {
+    float4 x[MLP_NV];
+    float z[MLP_NV];
+#pragma unroll
+    for (int i = 0; i < MLP_NV; ++i) {
+      const int64_t v = base + i * MLP_T + threadIdx.x;
+      x[i] = v < n ? X[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    mlp_z<MLP_NV>(su, b2, x, z);
+#pragma unroll
+    for (int i = 0; i < MLP_NV; ++i) {
+      const int64_t v = base + i * MLP_T + threadIdx.x;
+      if (v < n) gout[v] = mlp_g(z[i], rinfo[v]);
+    }
   }
 }
 
 // Loss and gradient, per-block partials (fixed order, deterministic).
-// Pass over tiles of MLP_T vertices: thread t runs the forward pass of vertex
-// t of the tile and its dL/dz; then thread j accumulates the gradient of
-// hidden unit j over the tile's vertices in order.
+// Pass over tiles of NV MLP_T vertices: a thread runs the forward pass of NV
+// vertices and their dL/dz; then warp w takes a quarter of the tile's vertices,
+// each lane the gradient of four hidden units, so that a load of a vertex's
+// features serves four units; the warps have sums of their own, added at the
+// end.  w2[j], the same factor in every
+// term of the hidden layer's gradient, is multiplied once at the end.
+constexpr int MLP_W = MLP_T / 32;
+constexpr int MLP_UL = HID / 32;  // hidden units per lane
+constexpr int GRAD_V = NF + 2;    // sums per hidden unit
+static_assert(HID == MLP_T, "a thread per hidden unit writes the partials");
+template <int NV>
 __global__ void __launch_bounds__(MLP_T) k_mlp_grad(int32_t n, const float4* __restrict__ X,
                                                     const uint4* __restrict__ rinfo, const float* __restrict__ y,
                                                     const float* __restrict__ params, float inv_n,
                                                     float* __restrict__ gpart, double* __restrict__ lpart) {
-  __shared__ __align__(16) float sw[NPARAM];
-  __shared__ float4 sx[MLP_T];
-  __shared__ float sdz[MLP_T];
+  constexpr int TILE = NV * MLP_T;
+  __shared__ Unit su[HID];
+  __shared__ float4 sx[TILE];
+  __shared__ float sdz[TILE];
+  __shared__ float sg[MLP_W][GRAD_V][HID];
+  __shared__ float sb[MLP_W];
   __shared__ double sl[MLP_T];
-  load_params(params, sw);
-  const int j = threadIdx.x;
-  float gW0 = 0.f, gW1 = 0.f, gW2 = 0.f, gW3 = 0.f, gb1 = 0.f, gw2 = 0.f, gb2 = 0.f;
+  load_params(params, su);
+  const float b2 = bf16r(params[OFF_B2]);
+  const int j = threadIdx.x, lane = j & 31, wid = j >> 5;
+  float4 w[MLP_UL], gW[MLP_UL];
+  float ub[MLP_UL], gb1[MLP_UL], gw2[MLP_UL];
+#pragma unroll
+  for (int q = 0; q < MLP_UL; ++q) {
+    w[q] = su[lane + 32 * q].w;
+    ub[q] = su[lane + 32 * q].b;
+    gW[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    gb1[q] = gw2[q] = 0.f;
+  }
+  float gb2 = 0.f;
   double lsum = 0.0;
-  const float* wj = sw + OFF_W1 + j * NF;
-  for (int64_t base = (int64_t)blockIdx.x * MLP_T; base < n; base += (int64_t)gridDim.x * MLP_T) {
-    const int64_t v = base + j;
-    float dz = 0.0f;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (v < n) {
-      x = X[v];
-      const float z = mlp_z(sw, x);
-      const float s = 1.0f / (1.0f + expf(-z));
-      const float p = (float)p_of(rinfo[v]);
-      const float g = p + (1.0f - p) * s;
-      const float r = g - y[v];
-      lsum += (double)r * (double)r;
-      dz = 2.0f * r * inv_n * (1.0f - p) * s * (1.0f - s);
+  for (int64_t base = (int64_t)blockIdx.x * TILE; base < n; base += (int64_t)gridDim.x * TILE) {
+    float4 x[NV];
+    float z[NV];
+    bool fin = true;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int64_t v = base + i * MLP_T + j;
+      x[i] = v < n ? X[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+      fin = fin && isfinite(x[i].x) && isfinite(x[i].y) && isfinite(x[i].z) && isfinite(x[i].w);
     }
-    sx[j] = x;
-    sdz[j] = dz;
-    __syncthreads();
-    const int cnt = (n - base) < (int64_t)MLP_T ? (int)(n - base) : MLP_T;
-    for (int i = 0; i < cnt; ++i) {
-      const float4 xi = sx[i];
-      const float dzi = sdz[i];
-      float pre = sw[OFF_B1 + j];
-      pre = fmaf(wj[0], xi.x, pre);
-      pre = fmaf(wj[1], xi.y, pre);
-      pre = fmaf(wj[2], xi.z, pre);
-      pre = fmaf(wj[3], xi.w, pre);
-      if (pre > 0.0f) {
-        gw2 = fmaf(dzi, pre, gw2);
-        const float dpre = dzi * sw[OFF_W2 + j];
-        gW0 = fmaf(dpre, xi.x, gW0);
-        gW1 = fmaf(dpre, xi.y, gW1);
-        gW2 = fmaf(dpre, xi.z, gW2);
-        gW3 = fmaf(dpre, xi.w, gW3);
-        gb1 += dpre;
+    mlp_z<NV>(su, b2, x, z);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int64_t v = base + i * MLP_T + j;
+      float dz = 0.f;
+      if (v < n) {
+        const float s = 1.0f / (1.0f + expf(-z[i]));
+        const float p = p_of(rinfo[v]);
+        const float g = p + (1.0f - p) * s;
+        const float r = g - y[v];
+        lsum += (double)r * (double)r;
+        dz = 2.0f * r * inv_n * (1.0f - p) * s * (1.0f - s);
       }
-      if (j == 0) gb2 += dzi;
+      sx[i * MLP_T + j] = x[i];
+      sdz[i * MLP_T + j] = dz;
+      gb2 += dz;
+    }
+    // an inactive unit contributes nothing even where a feature is infinite or
+    // NaN: tiles with such features mask them, the others only dL/dz
+    const bool mask = __syncthreads_or(!fin) != 0;
+    if (!mask) {
+#pragma unroll 4
+      for (int i = wid; i < TILE; i += MLP_W) {
+        const float4 xi = sx[i];
+        const float dzi = sdz[i];
+#pragma unroll
+        for (int q = 0; q < MLP_UL; ++q) {
+          const float pre = mlp_pre(w[q], ub[q], xi);
+          const float d = pre > 0.0f ? dzi : 0.0f;
+          gw2[q] = fmaf(d, fmaxf(pre, 0.0f), gw2[q]);
+          gW[q].x = fmaf(d, xi.x, gW[q].x);
+          gW[q].y = fmaf(d, xi.y, gW[q].y);
+          gW[q].z = fmaf(d, xi.z, gW[q].z);
+          gW[q].w = fmaf(d, xi.w, gW[q].w);
+          gb1[q] += d;
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int i = wid; i < TILE; i += MLP_W) {
+        const float4 xi = sx[i];
+        const float dzi = sdz[i];
+#pragma unroll
+        for (int q = 0; q < MLP_UL; ++q) {
+          const float pre = mlp_pre(w[q], ub[q], xi);
+          if (!(pre > 0.0f)) continue;
+          gw2[q] = fmaf(dzi, pre, gw2[q]);
+          gW[q].x = fmaf(dzi, xi.x, gW[q].x);
+          gW[q].y = fmaf(dzi, xi.y, gW[q].y);
+          gW[q].z = fmaf(dzi, xi.z, gW[q].z);
+          gW[q].w = fmaf(dzi, xi.w, gW[q].w);
+          gb1[q] += dzi;
+        }
+      }
     }
     __syncthreads();
   }
+#pragma unroll
+  for (int q = 0; q < MLP_UL; ++q) {
+    const float s[GRAD_V] = {gW[q].x, gW[q].y, gW[q].z, gW[q].w, gb1[q], gw2[q]};
+#pragma unroll
+    for (int f = 0; f < GRAD_V; ++f) sg[wid][f][lane + 32 * q] = s[f];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) gb2 += __shfl_xor_sync(0xffffffffu, gb2, o);
+  if (lane == 0) sb[wid] = gb2;
+  sl[j] = lsum;
+  __syncthreads();
   // parameter-major partials: gpart[i * nb + block] (the reduction reads
   // each parameter's partials contiguously)
   const size_t nb = gridDim.x, b = blockIdx.x;
-  gpart[(size_t)(OFF_W1 + j * NF + 0) * nb + b] = gW0;
-  gpart[(size_t)(OFF_W1 + j * NF + 1) * nb + b] = gW1;
-  gpart[(size_t)(OFF_W1 + j * NF + 2) * nb + b] = gW2;
-  gpart[(size_t)(OFF_W1 + j * NF + 3) * nb + b] = gW3;
-  gpart[(size_t)(OFF_B1 + j) * nb + b] = gb1;
-  gpart[(size_t)(OFF_W2 + j) * nb + b] = gw2;
-  if (j == 0) gpart[(size_t)OFF_B2 * nb + b] = gb2;
-  sl[j] = lsum;
-  __syncthreads();
+  const float w2 = su[j].w2;
+#pragma unroll
+  for (int f = 0; f < GRAD_V; ++f) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < MLP_W; ++q) s += sg[q][f][j];
+    const int at = f < NF ? OFF_W1 + j * NF + f : f == NF ? OFF_B1 + j : OFF_W2 + j;
+    gpart[(size_t)at * nb + b] = f <= NF ? w2 * s : s;
+  }
+  if (j == 0) {
+    float s = 0.f;
+    for (int q = 0; q < MLP_W; ++q) s += sb[q];
+    gpart[(size_t)OFF_B2 * nb + b] = s;
+  }
   for (int s = MLP_T / 2; s > 0; s >>= 1) {
     if (j < s) sl[j] += sl[j + s];
     __syncthreads();
@@ -221,34 +363,33 @@ __global__ void __launch_bounds__(MLP_T) k_mlp_grad(int32_t n, const float4* __r
   if (j == 0) lpart[blockIdx.x] = sl[0];
 }
 
-// One block per parameter (block NPARAM: the loss): the block's threads sum
-// strided runs of the partials, then a fixed-order tree in shared memory, so
-// the result is deterministic.  out = (accumulate ? out : 0) + weight * sum.
-constexpr int RED_T = 256;
+// One warp per parameter (warp NPARAM: the loss): the lanes sum strided runs of
+// the partials, then a fixed-order tree of shuffles, so the result is
+// deterministic.  out = (accumulate ? out : 0) + weight * sum.
+constexpr int RED_T = 128;
 __global__ void __launch_bounds__(RED_T) k_mlp_grad_reduce(const float* __restrict__ gpart,
                                                            const double* __restrict__ lpart, int nb, double inv_n,
                                                            float weight, int accumulate, float* __restrict__ grad,
                                                            float* __restrict__ loss) {
-  __shared__ double red[RED_T];
-  const int i = blockIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int i = (int)(blockIdx.x * (RED_T / 32) + (threadIdx.x >> 5));
+  if (i > NPARAM) return;
   double s = 0.0;
   if (i < NPARAM) {
-    for (int b = threadIdx.x; b < nb; b += RED_T) s += (double)gpart[(size_t)i * nb + b];
+#pragma unroll 8
+    for (int b = lane; b < nb; b += 32) s += (double)gpart[(size_t)i * nb + b];
   } else {
-    for (int b = threadIdx.x; b < nb; b += RED_T) s += lpart[b];
+#pragma unroll 8
+    for (int b = lane; b < nb; b += 32) s += lpart[b];
   }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = RED_T / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x != 0) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane != 0) return;
   if (i < NPARAM) {
-    const float v = weight * (float)red[0];
+    const float v = weight * (float)s;
     grad[i] = accumulate ? grad[i] + v : v;
   } else if (loss != nullptr) {
-    const float v = weight * (float)(red[0] * inv_n);
+    const float v = weight * (float)(s * inv_n);
     *loss = accumulate ? *loss + v : v;
   }
 }
@@ -266,9 +407,12 @@ __global__ void k_adam(int32_t count, float* __restrict__ params, const float* _
   params[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-static int mlp_blocks(int32_t n) {
-  int64_t b = ((int64_t)n + MLP_T - 1) / MLP_T;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(b, 152 * 8));
+// Blocks for n vertices in tiles of `tile`: at most eight per SM, with equal
+// numbers of tiles.
+static int mlp_blocks(int32_t n, int tile) {
+  const int64_t tiles = ((int64_t)n + tile - 1) / tile;
+  const int64_t per = (tiles + 152 * 8 - 1) / (152 * 8);
+  return (int)((tiles + per - 1) / per);
 }
 
 }  // namespace fcx
@@ -286,10 +430,11 @@ extern "C" fc_status fc_vertex_features(fc_graph* g, int32_t alpha_idx, float* X
   unsigned long long* s2 = nullptr;
   FC_CK(cudaMallocAsync((void**)&s2, (size_t)g->n * sizeof(unsigned long long), st));
   FC_CK(cudaMemsetAsync(s2, 0, (size_t)g->n * sizeof(unsigned long long), st));
-  const int64_t chunks = (g->nnz + NDS_CHUNK - 1) / NDS_CHUNK;  // one warp each, 8 warps per block
-  if (chunks > 0) {
-    const unsigned nb = (unsigned)std::min<int64_t>((chunks + 7) / 8, 152 * 8);
-    k_nbr_deg_sum<<<nb, 256, 0, st>>>(g->n, g->nnz, g->rowptr, g->colidx, g->deg, s2);
+  const int64_t tiles = (g->nnz + NDS_TILE - 1) / NDS_TILE;
+  if (tiles > 0) {
+    const int64_t per = (tiles + 152 * 6 - 1) / (152 * 6);  // consecutive tiles per block, six blocks per SM
+    k_nbr_deg_sum<<<(unsigned)((tiles + per - 1) / per), NDS_T, 0, st>>>(g->n, g->nnz, g->rowptr, g->colidx, g->deg,
+                                                                         per, s2);
     FC_LAUNCHED();
   }
   const unsigned fb = (unsigned)std::min<int64_t>(((int64_t)g->n + 255) / 256, 152 * 16);
@@ -307,7 +452,7 @@ extern "C" fc_status fc_mlp_forward(fc_graph* g, int32_t alpha_idx, const float*
     return FC_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  k_mlp_forward<<<mlp_blocks(g->n), MLP_T, 0, st>>>(g->n, (const float4*)X, g->rowinfo + (size_t)alpha_idx * g->n,
+  k_mlp_forward<<<mlp_blocks(g->n, MLP_NV * MLP_T), MLP_T, 0, st>>>(g->n, (const float4*)X, g->rowinfo + (size_t)alpha_idx * g->n,
                                                     params, g_out);
   FC_LAUNCHED();
   return FC_OK;
@@ -322,15 +467,21 @@ extern "C" fc_status fc_mlp_loss_grad_acc(fc_graph* g, int32_t alpha_idx, const 
     return FC_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  const int nb = mlp_blocks(g->n);
+  // vertices per thread: the most that still gives every SM two blocks (GB300,
+  // whole calls with 1, 2, 4 vertices: n = 2^16 24, 27, - us; 2^17 37, 29, 34;
+  // 2^18 54, 45, 42; 2^22 -, 425, 397)
+  int nv = 4;
+  while (nv > 1 && g->n < (int64_t)152 * 2 * nv * MLP_T) nv /= 2;
+  const int nb = mlp_blocks(g->n, nv * MLP_T);
   float* gpart = nullptr;
   double* lpart = nullptr;
   FC_CK(cudaMallocAsync((void**)&gpart, (size_t)nb * NPARAM * sizeof(float), st));
   FC_CK(cudaMallocAsync((void**)&lpart, (size_t)nb * sizeof(double), st));
-  k_mlp_grad<<<nb, MLP_T, 0, st>>>(g->n, (const float4*)X, g->rowinfo + (size_t)alpha_idx * g->n, y, params,
+  (nv == 4 ? k_mlp_grad<4> : nv == 2 ? k_mlp_grad<2> : k_mlp_grad<1>)<<<nb, MLP_T, 0, st>>>(
+      g->n, (const float4*)X, g->rowinfo + (size_t)alpha_idx * g->n, y, params,
                                    1.0f / (float)g->n, gpart, lpart);
   FC_LAUNCHED();
-  k_mlp_grad_reduce<<<NPARAM + 1, RED_T, 0, st>>>(gpart, lpart, nb, 1.0 / (double)g->n, weight, accumulate ? 1 : 0,
+  k_mlp_grad_reduce<<<(NPARAM + RED_T / 32) / (RED_T / 32), RED_T, 0, st>>>(gpart, lpart, nb, 1.0 / (double)g->n, weight, accumulate ? 1 : 0,
                                                   grad, loss);
   FC_LAUNCHED();
   FC_CK(cudaFreeAsync(gpart, st));
