@@ -101,9 +101,11 @@ __global__ void k_correct(int32_t n, const double* __restrict__ scal, const floa
   const int j = blockIdx.y;
   const double* sc = scal + j * 8;
   if (sc[5] == 0.0) return;
+  const double f = 1.0 / sc[4];  // one division per thread: GB300's FP64 rate is low (n = 2.1M: 90 us
+  // with a division per entry)
   const size_t off = (size_t)j * n;
   for (int64_t v = (int64_t)blockIdx.x * SV_T + threadIdx.x; v < n; v += (int64_t)gridDim.x * SV_T)
-    x[off + v] += (double)d[off + v] / sc[4];
+    x[off + v] += (double)d[off + v] * f;
 }
 
 // the FP32 diagonal and its reciprocal (the Jacobi preconditioner, applied
@@ -125,8 +127,17 @@ __global__ void k_fill(int64_t len, double val, double* __restrict__ a) {
 
 // x over V' (n+1 entries, x[n] = x(u*) = 0 on entry) -> mean-zero gauge
 __global__ void k_shift(int64_t len, const double* __restrict__ sum, double* __restrict__ x) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < len) x[i] -= *sum / (double)len;
+  const double mean = *sum / (double)len;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
+    x[i] -= mean;
+}
+
+// *any = 1 where an entry differs from zero
+__global__ void k_any_nonzero(int64_t len, const double* __restrict__ x, uint32_t* __restrict__ any) {
+  bool nz = false;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
+    nz |= x[i] != 0.0;
+  if (__syncthreads_or(nz) && threadIdx.x == 0) atomicOr(any, 1u);
 }
 
 __global__ void k_partial_sum(int64_t len, const double* __restrict__ a, double* __restrict__ part) {
@@ -538,14 +549,15 @@ __global__ void __launch_bounds__(SV_T) k_tile_rowsum64(TileArgs<double> a, cons
             sm.off[threadIdx.x >> 5]);
 }
 
-// r = b - (sigma + alpha d_w) x + alpha s; partial sums of r.r and b.b
+// r = b - (sigma + alpha d_w) x + alpha s (r = b when x is zero); partial sums
+// of r.r and b.b
 __global__ void __launch_bounds__(SV_T) k_resid_rows(int32_t n, TileArgs<double> a, const double* __restrict__ dw,
                                                      double sigma, double alpha, const double* __restrict__ b,
                                                      const double* __restrict__ x, double* __restrict__ r,
-                                                     double* __restrict__ prr, double* __restrict__ pbb) {
+                                                     double* __restrict__ prr, double* __restrict__ pbb, bool zero) {
   double rr = 0.0, bb = 0.0;
   for (int64_t v = (int64_t)blockIdx.x * SV_T + threadIdx.x; v < n; v += (int64_t)gridDim.x * SV_T) {
-    const double ax = x[v] * (sigma + alpha * dw[v]) - alpha * row_total(a, v);
+    const double ax = zero ? 0.0 : x[v] * (sigma + alpha * dw[v]) - alpha * row_total(a, v);
     const double rv = b[v] - ax;
     r[v] = rv;
     rr += rv * rv;
@@ -796,6 +808,23 @@ __device__ __forceinline__ void il_store(T* p, const T (&x)[VW]) {
   for (int c = 0; c < VW; ++c) s[c] = x[c];
   *reinterpret_cast<typename ILVec<T, VW>::type*>(p) = v;
 }
+// the same, leaving L2 first: vectors that are only streamed, so that the
+// gathered one stays
+template <typename T, int VW>
+__device__ __forceinline__ void il_load_s(const T* p, T (&x)[VW]) {
+  const auto v = __ldcs(reinterpret_cast<const typename ILVec<T, VW>::type*>(p));
+  const T* s = reinterpret_cast<const T*>(&v);
+#pragma unroll
+  for (int c = 0; c < VW; ++c) x[c] = s[c];
+}
+template <typename T, int VW>
+__device__ __forceinline__ void il_store_s(T* p, const T (&x)[VW]) {
+  typename ILVec<T, VW>::type v;
+  T* s = reinterpret_cast<T*>(&v);
+#pragma unroll
+  for (int c = 0; c < VW; ++c) s[c] = x[c];
+  __stcs(reinterpret_cast<typename ILVec<T, VW>::type*>(p), v);
+}
 
 // per-column sums over the block's rows to pa (and pb), fixed order
 template <int VW>
@@ -876,22 +905,21 @@ __device__ __forceinline__ void il_seg_sum(const int4& s, const int32_t* __restr
   for (int b = 0; b < s.y; b += PACK ? IL_U : 32) {
     const int left = min(PACK ? IL_U : 32, s.y - b);
     int32_t cj = 0;
-    float wj = 0.0f;
+    T wj = (T)0;  // (converted before the broadcast: once per entry, not once per lane)
     if (!PACK && (int)threadIdx.x < left) {
       cj = __ldg(colidx + e0 + b + threadIdx.x);
-      wj = w ? __ldg(w + e0 + b + threadIdx.x) : 1.0f;
+      wj = w ? (T)__ldg(w + e0 + b + threadIdx.x) : (T)1;
     }
     for (int k = 0; k < left; k += IL_U) {
-      T xv[IL_U][VW];
-      float ww[IL_U];
+      T xv[IL_U][VW], ww[IL_U];
 #pragma unroll
       for (int u = 0; u < IL_U; ++u) {
         int32_t c = 0;
-        ww[u] = 0.0f;
+        ww[u] = (T)0;
         if (PACK) {
           if (u < left) {
             c = __ldg(colidx + e0 + b + u);
-            ww[u] = w ? __ldg(w + e0 + b + u) : 1.0f;
+            ww[u] = w ? (T)__ldg(w + e0 + b + u) : (T)1;
           }
         } else {
           c = __shfl_sync(0xffffffffu, cj, (k + u) & 31);
@@ -907,29 +935,37 @@ __device__ __forceinline__ void il_seg_sum(const int4& s, const int32_t* __restr
       for (int u = 0; u < IL_U; ++u) {
         if (k + u < left) {
 #pragma unroll
-          for (int q = 0; q < VW; ++q) acc[q] += (T)ww[u] * xv[u][q];
+          for (int q = 0; q < VW; ++q) acc[q] += ww[u] * xv[u][q];
         }
       }
     }
   }
 }
 
-// [m][n] (column-major) <-> [n][m] (interleaved) through 32 x 32 tiles
-__global__ void k_il_transpose(int64_t rows, int64_t cols, const double* __restrict__ src, double* __restrict__ dst) {
+// dst[c ldd + i] = src[i lds + c] for i < rows, c < cols through 32 x 32 tiles:
+// column-major [m][n] <-> interleaved [n][m].  *any (or null) = 1 where an entry
+// differs from zero.
+__global__ void k_il_transpose(int64_t rows, int64_t cols, const double* __restrict__ src, int64_t lds,
+                               double* __restrict__ dst, int64_t ldd, uint32_t* __restrict__ any) {
   __shared__ double t[32][33];
+  bool nz = false;
   for (int64_t br = blockIdx.y; br * 32 < rows; br += gridDim.y)
     for (int64_t bc = blockIdx.x; bc * 32 < cols; bc += gridDim.x) {
       for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int64_t i = br * 32 + r, c = bc * 32 + threadIdx.x;
-        if (i < rows && c < cols) t[r][threadIdx.x] = src[i * cols + c];
+        if (i < rows && c < cols) {
+          t[r][threadIdx.x] = src[i * lds + c];
+          nz |= t[r][threadIdx.x] != 0.0;
+        }
       }
       __syncthreads();
       for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int64_t c = bc * 32 + r, i = br * 32 + threadIdx.x;
-        if (i < rows && c < cols) dst[c * rows + i] = t[threadIdx.x][r];
+        if (i < rows && c < cols) dst[c * ldd + i] = t[threadIdx.x][r];
       }
       __syncthreads();
     }
+  if (any && __syncthreads_or(nz) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(any, 1u);
 }
 
 // r = b - (sigma + alpha d_w) x + alpha s of one row
@@ -955,12 +991,14 @@ __global__ void __launch_bounds__(IL_T) k_il_resid(int m, int nseg, const int4* 
                                                   const double* __restrict__ dw, double sigma, double alpha,
                                                   const double* __restrict__ b, const double* __restrict__ x,
                                                   double* __restrict__ r, double* __restrict__ plong,
-                                                  double* __restrict__ prr, double* __restrict__ pbb, int nb) {
+                                                  double* __restrict__ prr, double* __restrict__ pbb, int nb,
+                                                  bool zero) {
   const int j0 = (int)(blockIdx.y * blockDim.x + threadIdx.x) * VW;
   const bool on = j0 < m;
   double rr[VW] = {}, bb[VW] = {};
   for (int g = blockIdx.x * blockDim.y + threadIdx.y; g < nseg; g += gridDim.x * blockDim.y) {
-    const int4 s = segs[g];
+    int4 s = segs[g];
+    if (zero) s.y = 0;  // x = 0: no products
     double acc[VW];
     il_seg_sum<double, VW, PACK>(s, colidx, w, x, m, j0, on, acc);
     if (!on) continue;
@@ -1043,7 +1081,7 @@ __device__ __forceinline__ void il_spmv_row(size_t i, float dg, float alpha, con
     qv[c] = pv[c] * dg - alpha * acc[c];
     pq[c] = fmaf(pv[c], qv[c], pq[c]);
   }
-  il_store<float, VW>(in.q + i, qv);
+  il_store_s<float, VW>(in.q + i, qv);
 }
 
 // q = A p, partials of p.q
@@ -1112,8 +1150,8 @@ __global__ void __launch_bounds__(IL_T) k_il_update(int32_t n, int m, const floa
     for (int u = 0; u < IL_V; ++u) {
       if (v0 + u < n) {
         const size_t i = (size_t)(v0 + u) * m + j0;
-        il_load<float, VW>(in.r + i, r[u]);
-        il_load<float, VW>(in.q + i, q[u]);
+        il_load_s<float, VW>(in.r + i, r[u]);
+        il_load_s<float, VW>(in.q + i, q[u]);
         pr[u] = prec ? prec[v0 + u] : 1.0f;
       }
     }
@@ -1126,7 +1164,7 @@ __global__ void __launch_bounds__(IL_T) k_il_update(int32_t n, int m, const floa
           rz[c] = fmaf(r[u][c], r[u][c] * pr[u], rz[c]);
           rr[c] = fmaf(r[u][c], r[u][c], rr[c]);
         }
-        il_store<float, VW>(in.r + (size_t)(v0 + u) * m + j0, r[u]);
+        il_store_s<float, VW>(in.r + (size_t)(v0 + u) * m + j0, r[u]);
       }
     }
   }
@@ -1158,9 +1196,9 @@ __global__ void __launch_bounds__(IL_T) k_il_p(int32_t n, int m, const float* __
     for (int u = 0; u < IL_V; ++u) {
       if (v0 + u < n) {
         const size_t i = (size_t)(v0 + u) * m + j0;
-        il_load<float, VW>(in.r + i, r[u]);
+        il_load_s<float, VW>(in.r + i, r[u]);
         il_load<float, VW>(in.p + i, p[u]);
-        il_load<float, VW>(in.d + i, d[u]);
+        il_load_s<float, VW>(in.d + i, d[u]);
         pr[u] = prec ? prec[v0 + u] : 1.0f;
       }
     }
@@ -1173,7 +1211,7 @@ __global__ void __launch_bounds__(IL_T) k_il_p(int32_t n, int m, const float* __
           d[u][c] += a[c] * p[u][c];
           p[u][c] = r[u][c] * pr[u] + beta[c] * p[u][c];
         }
-        il_store<float, VW>(in.d + i, d[u]);
+        il_store_s<float, VW>(in.d + i, d[u]);
         il_store<float, VW>(in.p + i, p[u]);
       }
     }
@@ -1199,53 +1237,50 @@ __global__ void __launch_bounds__(IL_T) k_il_correct(int32_t n, int m, const dou
   }
 }
 
-// Per-column scalars after the products: pq and a = rz / pq (a block per
-// column, fixed order).
-__global__ void __launch_bounds__(128) k_il_alpha(const double* __restrict__ ppq, int nb, double* __restrict__ scal) {
-  __shared__ double red[128];
-  const int j = blockIdx.x;
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nb; i += 128) s += ppq[(size_t)j * nb + i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = 64; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
+// sum of part[0..nb) by one warp, fixed order, valid in every lane
+__device__ __forceinline__ double il_warp_sum(const double* __restrict__ part, int nb) {
+  double s[4] = {};
+  for (int i = threadIdx.x & 31; i < nb; i += 128) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + 32 * k < nb) s[k] += part[i + 32 * k];
   }
-  if (threadIdx.x == 0) {
+  double x = (s[0] + s[2]) + (s[1] + s[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Per-column scalars after the products: pq and a = rz / pq (a warp per column;
+// a block per column took 19 us for 4096 columns; 2176 take 8 now).
+constexpr int IL_SW = 4;  // warps per block
+__global__ void __launch_bounds__(32 * IL_SW) k_il_alpha(int m, const double* __restrict__ ppq, int nb,
+                                                        double* __restrict__ scal) {
+  const int j = blockIdx.x * IL_SW + (threadIdx.x >> 5);
+  if (j >= m) return;
+  const double pq = il_warp_sum(ppq + (size_t)j * nb, nb);
+  if ((threadIdx.x & 31) == 0) {
     double* sc = scal + (size_t)j * 8;
-    sc[1] = red[0];
-    sc[6] = (sc[5] != 0.0 && red[0] != 0.0) ? sc[0] / red[0] : 0.0;
+    sc[1] = pq;
+    sc[6] = (sc[5] != 0.0 && pq != 0.0) ? sc[0] / pq : 0.0;
   }
 }
 
 // After the update: the new r.z and r.r, beta = rz_new / rz, rz <- rz_new.
-__global__ void __launch_bounds__(128) k_il_beta(const double* __restrict__ prz, const double* __restrict__ prr, int nb,
-                                                 double* __restrict__ scal, double* __restrict__ rr_out) {
-  __shared__ double ra[128], rb[128];
-  const int j = blockIdx.x;
-  double s = 0.0, t = 0.0;
-  for (int i = threadIdx.x; i < nb; i += 128) {
-    s += prz[(size_t)j * nb + i];
-    t += prr[(size_t)j * nb + i];
-  }
-  ra[threadIdx.x] = s;
-  rb[threadIdx.x] = t;
-  __syncthreads();
-  for (int k = 64; k > 0; k >>= 1) {
-    if (threadIdx.x < k) {
-      ra[threadIdx.x] += ra[threadIdx.x + k];
-      rb[threadIdx.x] += rb[threadIdx.x + k];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
+__global__ void __launch_bounds__(32 * IL_SW) k_il_beta(int m, const double* __restrict__ prz,
+                                                       const double* __restrict__ prr, int nb,
+                                                       double* __restrict__ scal, double* __restrict__ rr_out) {
+  const int j = blockIdx.x * IL_SW + (threadIdx.x >> 5);
+  if (j >= m) return;
+  const double rz = il_warp_sum(prz + (size_t)j * nb, nb);
+  const double rr = il_warp_sum(prr + (size_t)j * nb, nb);
+  if ((threadIdx.x & 31) == 0) {
     double* sc = scal + (size_t)j * 8;
-    sc[7] = sc[0] != 0.0 ? ra[0] / sc[0] : 0.0;
-    sc[0] = ra[0];
-    sc[2] = ra[0];
-    sc[3] = rb[0];
-    rr_out[j] = rb[0];
+    sc[7] = sc[0] != 0.0 ? rz / sc[0] : 0.0;
+    sc[0] = rz;
+    sc[2] = rz;
+    sc[3] = rr;
+    rr_out[j] = rr;
   }
 }
 
@@ -1261,12 +1296,12 @@ struct ILPlan {
 
 template <int VW>
 static void il_launch_resid(const ILPlan& pl, const fc_graph* g, int m, double sigma, double alpha, const double* b,
-                            const double* x, double* r, double* pA, double* pB, cudaStream_t st) {
+                            const double* x, double* r, double* pA, double* pB, bool zero, cudaStream_t st) {
   const dim3 blk(pl.lw, IL_T / pl.lw);
   const int nb = pl.gxs + pl.gxl;
   auto* kern = pl.lw == 32 ? k_il_resid<VW, false> : k_il_resid<VW, true>;
   kern<<<dim3(pl.gxs, pl.gy), blk, 0, st>>>(m, pl.nseg, pl.segs, g->colidx, g->w, g->dw, sigma, alpha, b, x, r,
-                                            (double*)pl.plong, pA, pB, nb);
+                                            (double*)pl.plong, pA, pB, nb, zero);
   note_launch();
   if (pl.nlong > 0) {
     k_il_long_resid<VW><<<dim3(pl.gxl, pl.gy), blk, 0, st>>>(m, pl.nlong, pl.longs, g->dw, sigma, alpha, b, x, r,
@@ -1297,9 +1332,9 @@ static void il_launch_iter(const ILPlan& pl, const fc_graph* g, int m, const flo
                                                             (const float*)pl.plong, pA, nb, pl.gxs);
     note_launch();
   }
-  k_il_alpha<<<m, 128, 0, st>>>(pA, nb, scal);
+  k_il_alpha<<<(m + IL_SW - 1) / IL_SW, 32 * IL_SW, 0, st>>>(m, pA, nb, scal);
   k_il_update<VW><<<dim3(pl.gxe, pl.gy), blk, 0, st>>>(g->n, m, prec, scal, in, pA, pB, pl.gxe);
-  k_il_beta<<<m, 128, 0, st>>>(pA, pB, pl.gxe, scal, rr_out);
+  k_il_beta<<<(m + IL_SW - 1) / IL_SW, 32 * IL_SW, 0, st>>>(m, pA, pB, pl.gxe, scal, rr_out);
   k_il_p<VW><<<dim3(pl.gxe, pl.gy), blk, 0, st>>>(g->n, m, prec, scal, in);
   for (int i = 0; i < 5; ++i) note_launch();
 }
@@ -1331,7 +1366,13 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     return FC_EINVAL;
   }
   const int32_t n = g->n;
-  const int m = n_rhs;
+  // values per lane: a warp takes up to 64 columns, and 128 in 16-byte accesses
+  // from 128 on.  The columns are filled up with zero columns (never active) to a
+  // multiple of them (R-MAT 2^16: 33 columns 12.9 ms, 63 17.6 -> 13.4 against one
+  // value per lane; 96 columns 19.7 with two values, 21.6 with four; filling up
+  // to 8 or 16 columns changes less than 5% either way)
+  const int vw = n_rhs >= 128 ? 4 : n_rhs > 32 ? 2 : 1, pad = vw - 1;
+  const int m = n_rhs + pad <= 65535 ? (n_rhs + pad) & ~pad : n_rhs;
   const double alpha = g->alphas[alpha_idx];
   const int nb = (n + SV_T - 1) / SV_T;  // blocks of the element-wise kernels
   const size_t nm = (size_t)n * m;
@@ -1358,7 +1399,22 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   void* seg_mem = nullptr;
   void* plong = nullptr;
   const int gy = (m + 31) / 32;  // column tiles of the transposes
+  uint32_t* any = nullptr;       // x differs from zero on entry
+  uint32_t h_any = 1;
+  FC_CK(cudaMallocAsync((void**)&any, 4, st));
+  FC_CK(cudaMemsetAsync(any, 0, 4, st));
   if (il) {
+    FC_CK(cudaMallocAsync((void**)&bi, nm * sizeof(double), st));
+    FC_CK(cudaMallocAsync((void**)&xi, nm * sizeof(double), st));
+    if (m != n_rhs) {
+      FC_CK(cudaMemsetAsync(bi, 0, nm * sizeof(double), st));
+      FC_CK(cudaMemsetAsync(xi, 0, nm * sizeof(double), st));
+    }
+    const dim3 tg((unsigned)std::min<int64_t>((n + 31) / 32, 1024), (unsigned)std::min<int64_t>(gy, 1024));
+    k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(n_rhs, n, b, n, bi, m, nullptr);
+    FC_LAUNCHED();
+    k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(n_rhs, n, x, n, xi, m, any);
+    FC_LAUNCHED();
     // row segments (k_il_seg_count, _fill)
     const int len = m > 16 ? IL_SEG : IL_SEG_PACK;
     const size_t n1 = (size_t)n + 1, lmax = (size_t)(g->nnz / len) + 1, smax = (size_t)n + lmax;
@@ -1379,6 +1435,7 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     FC_CK(cudaMemcpyAsync(h, off + n, 4, cudaMemcpyDeviceToHost, st));
     FC_CK(cudaMemcpyAsync(h + 1, loff + n, 4, cudaMemcpyDeviceToHost, st));
     FC_CK(cudaMemcpyAsync(h + 2, lidx + n, 4, cudaMemcpyDeviceToHost, st));
+    FC_CK(cudaMemcpyAsync(&h_any, any, 4, cudaMemcpyDeviceToHost, st));
     FC_CK(cudaStreamSynchronize(st));
     FC_CK(cudaMallocAsync(&plong, std::max<size_t>(1, (size_t)h[1] * m * sizeof(double)), st));
     int nsm = 0;
@@ -1405,17 +1462,8 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
       npart = std::max(npart, std::max(p.gxs + p.gxl, p.gxe));
       return p;
     };
-    // values per lane: 16-byte accesses where the columns divide evenly and a
-    // warp's columns are filled
-    il32 = plan(m % 4 == 0 && m >= 128 ? 4 : m % 2 == 0 && m >= 64 ? 2 : 1);
-    il64 = plan(m % 2 == 0 && m >= 64 ? 2 : 1);
-    FC_CK(cudaMallocAsync((void**)&bi, nm * sizeof(double), st));
-    FC_CK(cudaMallocAsync((void**)&xi, nm * sizeof(double), st));
-    const dim3 tg((unsigned)std::min<int64_t>((n + 31) / 32, 1024), (unsigned)std::min<int64_t>(gy, 1024));
-    k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(m, n, b, bi);
-    FC_LAUNCHED();
-    k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(m, n, x, xi);
-    FC_LAUNCHED();
+    il32 = plan(m % vw == 0 ? vw : 1);
+    il64 = plan(m % vw == 0 ? std::min(vw, 2) : 1);
   }
   const double* bv = il ? bi : b;
   double* xv = il ? xi : x;
@@ -1495,6 +1543,9 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     k_span_bits<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, g->rowptr, span, nempty);
     FC_LAUNCHED();
     uint32_t h_nempty = 1;
+    k_any_nonzero<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(n, x, any);
+    FC_LAUNCHED();
+    FC_CK(cudaMemcpyAsync(&h_any, any, 4, cudaMemcpyDeviceToHost, st));
     FC_CK(cudaMemcpyAsync(&h_nempty, nempty, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     FC_CK(cudaStreamSynchronize(st));
     fold = h_nempty == 0;
@@ -1509,16 +1560,17 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   int used = 0;
   fc_status result = FC_ENOCONV;
   for (int outer = 0; outer < 64; ++outer) {
+    const bool zero = outer == 0 && h_any == 0;  // x = 0: the residual is b
     const int nres = il ? il64.gxs + il64.gxl : nbx;  // residual partials per column
     if (il) {
-      if (il64.vw == 2) il_launch_resid<2>(il64, g, m, sigma, alpha, bv, xv, r64, pA, pB, st);
-      else il_launch_resid<1>(il64, g, m, sigma, alpha, bv, xv, r64, pA, pB, st);
+      if (il64.vw == 2) il_launch_resid<2>(il64, g, m, sigma, alpha, bv, xv, r64, pA, pB, zero, st);
+      else il_launch_resid<1>(il64, g, m, sigma, alpha, bv, xv, r64, pA, pB, zero, st);
     } else {
-      if (ntiles > 0) {
+      if (ntiles > 0 && !zero) {
         k_tile_rowsum64<<<tile_grid, SV_T, 0, st>>>(t64, x, ntiles);
         FC_LAUNCHED();
       }
-      k_resid_rows<<<nbx, SV_T, 0, st>>>(n, t64, g->dw, sigma, alpha, b, x, r64, pA, pB);
+      k_resid_rows<<<nbx, SV_T, 0, st>>>(n, t64, g->dw, sigma, alpha, b, x, r64, pA, pB, zero);
     }
     FC_LAUNCHED();
     k_colsum<<<m, SV_T, 0, st>>>(pA, nres, sums);
@@ -1622,13 +1674,14 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   }
   if (il) {
     const dim3 tg((unsigned)std::min<int64_t>(gy, 1024), (unsigned)std::min<int64_t>((n + 31) / 32, 1024));
-    k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(n, m, xi, x);
+    k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(n, n_rhs, xi, m, x, n, nullptr);
     FC_LAUNCHED();
     FC_CK(cudaFreeAsync(bi, st));
     FC_CK(cudaFreeAsync(xi, st));
     FC_CK(cudaFreeAsync(seg_mem, st));
     FC_CK(cudaFreeAsync(plong, st));
   }
+  FC_CK(cudaFreeAsync(any, st));
   FC_CK(cudaFreeAsync(r64, st));
   FC_CK(cudaFreeAsync(f32, st));
   FC_CK(cudaFreeAsync(part, st));
@@ -1674,7 +1727,7 @@ extern "C" fc_status fc_pivot_solve(fc_graph* g, int32_t alpha_idx, double* x, d
   fcx::note_launch();
   k_colsum<<<1, SV_T, 0, st>>>(part, nb, part + nb);
   fcx::note_launch();
-  k_shift<<<(unsigned)((n1 + 255) / 256), 256, 0, st>>>(n1, part + nb, x);
+  k_shift<<<(unsigned)std::min<int64_t>((n1 + 255) / 256, 152 * 8), 256, 0, st>>>(n1, part + nb, x);
   FC_LAUNCHED();
   FC_CK(cudaFreeAsync(rhs, st));
   FC_CK(cudaFreeAsync(part, st));
