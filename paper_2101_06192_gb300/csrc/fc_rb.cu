@@ -19,9 +19,9 @@
 // takes a barrier per tree level, so deep trees cost no more barriers than
 // shallow ones: child counts (with validation); subtree sizes and sibling
 // offsets by peeling leaves (one atomic per tree node, the node finished by
-// whichever thread delivers its last child); preorder numbers by pointer
-// jumping down the paths (O(log depth) rounds); the rows; and the
-// per-vertex sums.  Preorder numbers and sizes are stored vertex-major
+// whichever thread delivers its last child); the roots' offsets; preorder
+// numbers by pointer jumping down the paths (O(log depth) rounds); and the rows
+// with the per-vertex sums.  Preorder numbers and sizes are stored vertex-major
 // across the chunk's trees, so a warp scanning a row with one lane per tree
 // reads each neighbour's numbers for all trees in one 128-byte line.  Long
 // unweighted rows are split into segments of 256 entries whose counts add
@@ -29,6 +29,17 @@
 // tree's weights in row order.  Every loop bound and every early exit is
 // read from global memory after a barrier, so all CTAs take the same path
 // through the barriers.
+//
+// Bound by latency: the atomic chains of the peeling and the neighbours' lines.
+// Measured on GB300, 32 trees of R-MAT n = 2^18, m = 16: whole call 1470 ->
+// 1160 us.  Phases (with a clock read at each barrier): counts 52 -> 35;
+// peeling 410 -> 265 (children and sizes in one word, sizes read from it in the
+// end, idle lanes fed from a ring instead of by searching bit masks); roots'
+// offsets 165 -> 45 (a block scan and an atomic per 1024 vertices instead of a
+// grid-wide scan of all nodes); jumping 220 -> 175 (four loads in flight, two
+// jumps per round); rows about 470 -> 440 (no loads for leaves, one-segment rows
+// finished at once).  Four CTAs per SM: with five, registers spill (1300 us);
+// 16 loads in flight or rows from a shared counter change nothing (1160, 1150).
 //
 // The same kernel, in its second mode, aggregates the effective resistances
 // r(u, v) between a pivot u and every vertex v (Sec. 3, insight (iii)) from
@@ -74,19 +85,14 @@ struct RBParams {
   uint64_t* acc;              // [n] fixed-point sums
   const int4* segs;           // row segments {v, entries, first entry (low, high word)}
   const uint32_t* nseg;       // number of segments
-  // scratch.  Per tree node flat index i = t (n + 1) + v, where v = n is the
-  // tree's u*; vertex-major index v Tc + t.
-  uint32_t* cnt;              // [Tc (n + 1)] children counts (zeroed by the host)
-  unsigned long long* word;   // [Tc (n + 1)] {summed sizes of finished children, finished children} (zeroed)
-  uint32_t* rsz;              // [Tc (n + 1)] subtree size of each root, 0 elsewhere
-  unsigned long long* jw;     // [Tc (n + 1)] pointer-jumping words {ancestor, partial preorder number}
+  // scratch.  Per tree node flat index i = t n + v; vertex-major index v Tc + t.
+  unsigned long long* word;   // [Tc n] {children not finished, summed sizes of the finished ones} (zeroed)
+  unsigned long long* jw;     // [Tc n] pointer-jumping words {ancestor, partial preorder number}
   int32_t* size;              // [n][Tc] subtree sizes (vertex-major)
   int32_t* tin;               // [n][Tc] preorder numbers (vertex-major)
-  double* sout;               // [n][Tc] weighted: sum over neighbours outside the subtree
-  uint32_t* outc;             // [n][Tc] unweighted: count of neighbours outside the subtree
-  uint32_t* rsum;             // [Tc (n + 1)] exclusive scan of the roots' subtree sizes
-  uint32_t* bsum;             // [gridDim.x] block totals of the scan
-  uint32_t* ctr;              // [2] error, [4..6] active counts of the jumping rounds, [7] chunk grabs (zeroed)
+  uint32_t* outc;             // [n][Tc] rows of several segments: count of neighbours outside the subtree
+  uint32_t* tsum;             // [Tc] vertices below the tree's roots so far (zeroed)
+  uint32_t* ctr;              // [2] error, [4..6] open flags of the jumping rounds, [7] chunk grabs (zeroed)
   const uint64_t* qtab;       // unweighted, one alpha: fixed-point value for each count of outside neighbours, or null
   // resistance mode
   int32_t root;               // the pivot u (the only child of u*), -1 in the diag(Omega) mode
@@ -124,111 +130,96 @@ __device__ __forceinline__ uint32_t block_exscan_u32(uint32_t x, uint32_t* total
   return ex;
 }
 
-// Grid-wide exclusive scan out[i] = sum_{j < i} val(j) (mod 2^32) over
-// [0, len): each CTA scans a contiguous range, CTA 0 scans the range totals,
-// and each CTA adds its carry.  Ends without a trailing barrier.
-template <class F>
-__device__ void grid_exscan(cg::grid_group& grid, F val, uint32_t* out, int64_t len, uint32_t* bsum,
-                            uint32_t* wsum, uint32_t* carry) {
-  const int64_t chunk = (len + gridDim.x - 1) / gridDim.x;
-  const int64_t b0 = std::min<int64_t>(len, (int64_t)blockIdx.x * chunk);
-  const int64_t b1 = std::min<int64_t>(len, b0 + chunk);
-  if (threadIdx.x == 0) *carry = 0;
-  __syncthreads();
-  for (int64_t base = b0; base < b1; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    const uint32_t x = i < b1 ? val(i) : 0u;
-    uint32_t tot = 0;
-    const uint32_t ex = block_exscan_u32(x, &tot, wsum);
-    if (i < b1) out[i] = *carry + ex;
-    __syncthreads();
-    if (threadIdx.x == 0) *carry += tot;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) bsum[blockIdx.x] = *carry;
-  grid.sync();
-  if (blockIdx.x == 0) {
-    if (threadIdx.x == 0) *carry = 0;
-    __syncthreads();
-    for (int base = 0; base < (int)gridDim.x; base += blockDim.x) {
-      const int j = base + threadIdx.x;
-      const uint32_t x = j < (int)gridDim.x ? bsum[j] : 0u;
-      uint32_t tot = 0;
-      const uint32_t ex = block_exscan_u32(x, &tot, wsum);
-      if (j < (int)gridDim.x) bsum[j] = *carry + ex;
-      __syncthreads();
-      if (threadIdx.x == 0) *carry += tot;
-      __syncthreads();
-    }
-  }
-  grid.sync();
-  const uint32_t add = bsum[blockIdx.x];
-  for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) out[i] += add;
-}
-
 __device__ __forceinline__ unsigned long long jw_pack(int32_t anc, int32_t sum) {
   return (unsigned long long)(uint32_t)anc | ((unsigned long long)(uint32_t)sum << 32);
 }
 
-constexpr int RB_TILE = 256;  // vertices per tile of the vertex-major transpose
+constexpr int RB_TILE = RB_T;  // vertices per tile of the vertex-major transpose
+
+__device__ __forceinline__ unsigned long long jw_load(const unsigned long long* p) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return w;
+}
+__device__ __forceinline__ void jw_store(unsigned long long* p, unsigned long long w) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+
+constexpr int RB_U = 4;               // nodes per thread and task: loads in flight
+constexpr int RB_CHUNK = RB_U * RB_T; // vertices of one tree per task
+constexpr int RB_RING = 64;           // leaves of a warp waiting for a lane
 
 // MODE 0: Rao-Blackwellised diag(Omega); MODE 1: effective resistances to the pivot.
 template <int MODE>
-__global__ void __launch_bounds__(RB_T, 5) k_rb(RBParams p) {
+__global__ void __launch_bounds__(RB_T, 4) k_rb(RBParams p) {
   cg::grid_group grid = cg::this_grid();
   __shared__ int32_t tile[RB_TMAX][RB_TILE + 1];
   __shared__ uint32_t wsum[32];
-  __shared__ uint32_t carry;
+  __shared__ uint32_t sbase;
   const int32_t n = p.n;
-  const int32_t n1 = n + 1;
   const int32_t Tc = p.Tc;
-  const int64_t N1 = (int64_t)Tc * n1;
+  const int64_t N = (int64_t)Tc * n;  // below 2^31
   const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
   const int lane = threadIdx.x & 31;
   const int64_t gwarp = gtid >> 5, nwarps = gstride >> 5;
 #define VT(t, v) ((int64_t)(v) * Tc + (t))
+  const int32_t chunks = (int32_t)(((int64_t)n + RB_CHUNK - 1) / RB_CHUNK);
+  // f(tree, flat index of its vertex 0, first vertex of the block) over this block's tasks
+  auto each = [&](auto f) {
+    for (int32_t task = blockIdx.x; task < Tc * chunks; task += gridDim.x) {
+      const int32_t t = task / chunks;
+      f(t, (int64_t)t * n, (uint32_t)(task - t * chunks) * RB_CHUNK);
+    }
+  };
 
   // ---- child counts; parents must lie in [0, n] and differ from the vertex ----
-  for (int64_t i = gtid; i < N1; i += gstride) {
-    const int32_t t = (int32_t)(i / n1), v = (int32_t)(i - (int64_t)t * n1);
-    p.rsz[i] = 0u;
-    if (v == n) {
-      p.jw[i] = jw_pack(-1, -1);
-      continue;
+  each([&](int32_t t, int64_t b, uint32_t c0) {
+#pragma unroll
+    for (int i = 0; i < RB_U; ++i) {
+      const uint32_t v = c0 + i * RB_T + threadIdx.x;
+      if (v >= (uint32_t)n) continue;
+      const int32_t par = p.parents[b + v];
+      if (par < 0 || par > n || par == (int32_t)v) atomicOr(&p.ctr[2], ERR_INVAL);
+      // a tree of G rooted at the pivot: the pivot, and only the pivot, hangs from u*
+      else if (MODE == 1 && ((par == n) != ((int32_t)v == p.root))) atomicOr(&p.ctr[2], ERR_INVAL);
+      else if (par < n) atomicAdd(&p.word[b + par], 1ull << 32);  // u*'s children: a scan below
     }
-    const int32_t par = p.parents[(int64_t)t * n + v];
-    if (par < 0 || par > n || par == v) atomicOr(&p.ctr[2], ERR_INVAL);
-    // a tree of G rooted at the pivot: the pivot, and only the pivot, hangs from u*
-    else if (MODE == 1 && ((par == n) != (v == p.root))) atomicOr(&p.ctr[2], ERR_INVAL);
-    else if (par < n) atomicAdd(&p.cnt[(int64_t)t * n1 + par], 1u);  // u*'s children: a scan below
-  }
+  });
   grid.sync();
   if (*(volatile uint32_t*)&p.ctr[2] != 0u) return;  // uniform: read after the barrier
 
   // ---- subtree sizes and sibling offsets by peeling leaves.  A finished
-  // child adds {its size, 1} to its parent's word in one atomic; the sizes
+  // child adds {-1, its size} to its parent's word in one atomic; the sizes
   // already there are its earlier-finished siblings', so 1 + that sum is its
   // offset in the parent's preorder interval (any sibling order gives valid
-  // intervals, and subtree membership does not depend on it).  The thread
-  // that delivers a parent's last child carries on with the parent: no
-  // barrier per tree level.  The roots (u*'s children, often most vertices)
-  // take their offsets from a scan instead of one contended word. ----
-  // Warps take candidates in chunks of 32 (coalesced, one chunk ahead)
-  // from a shared counter, eight chunks per grab, and hand the leaves among
-  // them to whichever lanes are idle.  The last deliverer of a node carries
-  // on with it, so chains pile up on some lanes; warps so held up take fewer
-  // chunks, and the rest of their lanes keep taking leaves.  A step loads the
-  // parent's child count and the grandparent before its atomic, so all three
-  // are in flight together.
+  // intervals, and subtree membership does not depend on it), and a node's
+  // size is 1 + the sum of its word in the end.  The thread that delivers a
+  // parent's last child carries on with the parent: no barrier per tree level.
+  // The roots (u*'s children, often most vertices) take their offsets below
+  // instead of from one contended word.  Warps take candidates in chunks of 32
+  // (coalesced, one chunk ahead) from a shared counter, eight chunks per grab,
+  // and put the leaves among them into a ring from which idle lanes take.  The
+  // last deliverer of a node carries on with it, so chains pile up on some
+  // lanes; warps so held up take fewer chunks.  A step loads the grandparent
+  // before its atomic, so both are in flight together. ----
   {
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t nchunks = (N1 + 31) / 32;
-    int64_t sc = 0;  // current grab (warp-uniform)
-    int kc = 8;      // next chunk within it
+    const int64_t nchunks = (N + 31) / 32;
+    int32_t* ring_v = &tile[0][0] + (threadIdx.x >> 5) * 3 * RB_RING;  // vertex, parent, flat index of the tree's vertex 0
+    int32_t* ring_p = ring_v + RB_RING;
+    int32_t* ring_b = ring_p + RB_RING;
+    unsigned head = 0, cnt = 0;  // warp-uniform
+    int64_t sc = 0;              // current grab (warp-uniform)
+    int kc = 8;                  // next chunk within it
     bool dry = false;
-    auto next_chunk = [&]() -> int64_t {
-      if (dry) return -1;
+    int32_t nb = 0, nv = 0, np = n;  // prefetched chunk: this lane's node
+    bool nleaf = false;
+    bool pre = false;  // a prefetched chunk is waiting (warp-uniform)
+    auto load = [&]() {
+      pre = false;
+      nleaf = false;
+      if (dry) return;
       if (kc == 8) {
         uint32_t g = 0;
         if (lane == 0) g = atomicAdd(&p.ctr[7], 1u);
@@ -236,119 +227,130 @@ __global__ void __launch_bounds__(RB_T, 5) k_rb(RBParams p) {
         kc = 0;
       }
       const int64_t c = sc * 8 + kc++;
-      if (c >= nchunks) dry = true;
-      return dry ? -1 : c;
-    };
-    int32_t nt = 0, nv = n, np = 0;  // prefetched chunk: this lane's node
-    uint32_t nc = 1u;
-    bool pre = false;  // a prefetched chunk is waiting (warp-uniform)
-    auto load = [&]() {
-      const int64_t c = next_chunk();
-      pre = c >= 0;
-      nt = 0;
-      nv = n;
-      nc = 1u;
-      np = 0;
-      const int64_t i = c * 32 + lane;
-      if (pre && i < N1) {
-        nt = (int32_t)(i / n1);
-        nv = (int32_t)(i - (int64_t)nt * n1);
-        if (nv != n) {
-          nc = p.cnt[i];
-          np = p.parents[(int64_t)nt * n + nv];
-        }
+      if (c >= nchunks) {
+        dry = true;
+        return;
+      }
+      pre = true;
+      const uint32_t i = (uint32_t)(c * 32) + lane;
+      if (i < (uint32_t)N) {
+        np = p.parents[i];
+        // (the word of a node whose children are all finished holds their sizes)
+        nleaf = *(volatile unsigned long long*)&p.word[i] == 0ull && np != n;
+        const uint32_t t = i / (uint32_t)n;
+        nb = (int32_t)(t * (uint32_t)n);
+        nv = (int32_t)i - nb;
       }
     };
     load();
-    unsigned lmask = 0;  // leaves of the current chunk not yet taken (warp-uniform)
-    int32_t ct = 0, cv = 0, cpar = 0;  // this lane's node of the current chunk
-    int32_t t = -1, v = 0, par = 0;
+    int32_t b = 0, v = -1, par = 0;  // this lane's node (none: v < 0)
     uint32_t s = 0;
     for (;;) {
-      if (lmask == 0u && pre) {  // the prefetched chunk becomes current
-        ct = nt;
-        cv = nv;
-        cpar = np;
-        lmask = __ballot_sync(0xffffffffu, nv != n && nc == 0u);
+      while (pre && cnt < 32u) {
+        const unsigned lm = __ballot_sync(0xffffffffu, nleaf);
+        if (nleaf) {
+          const unsigned at = (head + cnt + __popc(lm & lt)) & (RB_RING - 1);
+          ring_v[at] = nv;
+          ring_p[at] = np;
+          ring_b[at] = nb;
+        }
+        cnt += __popc(lm);
         load();
       }
-      const unsigned need = __ballot_sync(0xffffffffu, t < 0);
-      if (need == 0xffffffffu && lmask == 0u && !pre) break;  // uniform
-      const int avail = __popc(lmask);
-      const int ntake = min(__popc(need), avail);
-      const int r = __popc(need & lt);
-      const bool take = t < 0 && r < avail;
-      const int src = take ? (int)__fns(lmask, 0, r + 1) : lane;
-      const int32_t tt = __shfl_sync(0xffffffffu, ct, src);
-      const int32_t tv = __shfl_sync(0xffffffffu, cv, src);
-      const int32_t tp = __shfl_sync(0xffffffffu, cpar, src);
-      // the first ntake leaves are taken
-      lmask = ntake == avail ? 0u : lmask & ~((1u << __fns(lmask, 0, ntake + 1)) - 1u);
-      if (take) {
-        t = tt;
-        v = tv;
-        par = tp;
+      __syncwarp();
+      const unsigned need = __ballot_sync(0xffffffffu, v < 0);
+      if (need == 0xffffffffu && cnt == 0u) break;  // uniform (nothing prefetched: the loop above drained it)
+      const unsigned r = __popc(need & lt);
+      if (v < 0 && r < cnt) {
+        const unsigned at = (head + r) & (RB_RING - 1);
+        v = ring_v[at];
+        par = ring_p[at];
+        b = ring_b[at];
         s = 1u;
-        p.size[VT(t, v)] = 1;
       }
-      if (t < 0) continue;
-      if (par == n) {  // a root: its offset comes from the scan below
-        p.rsz[(int64_t)t * n1 + v] = s;
-        t = -1;
-        continue;
-      }
-      const int64_t pi = (int64_t)t * n1 + par;
-      const uint32_t cp = p.cnt[pi];
-      const int32_t gp = p.parents[(int64_t)t * n + par];
-      const unsigned long long old = atomicAdd(&p.word[pi], (1ull << 32) | s);
-      p.jw[(int64_t)t * n1 + v] = jw_pack((int32_t)pi, (int32_t)(1u + (uint32_t)old));
-      if ((uint32_t)(old >> 32) + 1u != cp) {
-        t = -1;
+      const unsigned took = min((unsigned)__popc(need), cnt);
+      head += took;
+      cnt -= took;
+      __syncwarp();
+      if (v < 0) continue;
+      const int32_t pi = b + par;
+      const int32_t gp = p.parents[pi];
+      const unsigned long long old = atomicAdd(&p.word[pi], (0xffffffffull << 32) | s);
+      p.jw[b + v] = jw_pack(pi, (int32_t)(1u + (uint32_t)old));
+      if ((uint32_t)(old >> 32) != 1u || gp == n) {
+        v = -1;
         continue;
       }
       s = 1u + (uint32_t)old + s;
       v = par;
       par = gp;
-      p.size[VT(t, v)] = (int32_t)s;
     }
   }
   grid.sync();
-  // roots in vertex order: preorder number = sizes of the tree's earlier roots
-  grid_exscan(grid, [&](int64_t i) { return p.rsz[i]; }, p.rsum, N1, p.bsum, wsum, &carry);
-  grid.sync();
-  for (int64_t i = gtid; i < N1; i += gstride) {
-    const int32_t t = (int32_t)(i / n1), v = (int32_t)(i - (int64_t)t * n1);
-    const uint32_t base = p.rsum[(int64_t)t * n1];
-    if (v == n) {
-      // a parent cycle leaves its vertices and their subtrees outside u*'s tree
-      if (p.rsum[i] - base != (uint32_t)n) atomicOr(&p.ctr[2], ERR_INVAL);
-    } else if (p.rsz[i] != 0u) {
-      p.jw[i] = jw_pack(-1, (int32_t)(p.rsum[i] - base));
+  // roots: preorder number = sizes of the tree's roots before it, by chunk in
+  // the order in which the blocks add up (any order of the roots will do)
+  each([&](int32_t t, int64_t b, uint32_t c0) {
+    uint32_t x[RB_U], s = 0;
+    bool root[RB_U];
+#pragma unroll
+    for (int i = 0; i < RB_U; ++i) {
+      const uint32_t v = c0 + i * RB_T + threadIdx.x;
+      root[i] = v < (uint32_t)n && p.parents[b + v] == n;
+      const unsigned long long w = root[i] ? *(volatile unsigned long long*)&p.word[b + v] : 0ull;
+      x[i] = s;
+      // (children left: the root of an unfinished tree, never in a forest)
+      s += root[i] && (w >> 32) == 0ull ? 1u + (uint32_t)w : 0u;
     }
-  }
+    uint32_t tot = 0;
+    const uint32_t ex = block_exscan_u32(s, &tot, wsum);
+    if (threadIdx.x == 0) sbase = tot ? atomicAdd(&p.tsum[t], tot) : 0u;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < RB_U; ++i)
+      if (root[i]) p.jw[b + c0 + i * RB_T + threadIdx.x] = jw_pack(-1, (int32_t)(sbase + ex + x[i]));
+    __syncthreads();
+  });
   grid.sync();
-  if (*(volatile uint32_t*)&p.ctr[2] != 0u) return;
+  // a parent cycle leaves its vertices and their subtrees outside u*'s tree
+  if (__syncthreads_or(threadIdx.x < Tc && *(volatile uint32_t*)&p.tsum[threadIdx.x] != (uint32_t)n)) {
+    if (gtid == 0) atomicOr(&p.ctr[2], ERR_INVAL);
+    return;  // uniform: every block reads the same sums
+  }
 
   // ---- preorder numbers: each node's number is its parent's plus its
-  // offset, summed down the path by pointer jumping.  Invariant: tin(i) =
-  // sum(i) + tin(anc(i)), with anc = -1 once sum is the number itself; words
-  // are read and written whole, so a node may read an ancestor's word of
-  // this round or the last one.  O(log depth) rounds. ----
+  // offset, summed down the path by pointer jumping, two jumps per round.
+  // Invariant: tin(i) = sum(i) + tin(anc(i)), with anc = -1 once sum is the
+  // number itself; words are read and written whole, so a node may read an
+  // ancestor's word of this round or the last one.  O(log depth) rounds. ----
   for (int r = 0;; ++r) {
-    uint32_t active = 0;
-    for (int64_t i = gtid; i < N1; i += gstride) {
-      volatile unsigned long long* jv = p.jw;
-      const unsigned long long w0 = jv[i];
-      const int32_t a = (int32_t)(uint32_t)w0;
-      if (a < 0) continue;
-      const unsigned long long w1 = jv[a];
-      const int32_t a1 = (int32_t)(uint32_t)w1;
-      jv[i] = jw_pack(a1, (int32_t)((uint32_t)(w0 >> 32) + (uint32_t)(w1 >> 32)));
-      active += a1 >= 0;
-    }
+    bool open = false;
+    each([&](int32_t t, int64_t b, uint32_t c0) {
+      unsigned long long w[RB_U], x[RB_U];
+      bool go[RB_U];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) active += __shfl_xor_sync(0xffffffffu, active, o);
-    if (lane == 0 && active) atomicAdd(&p.ctr[4 + r % 3], active);
+      for (int i = 0; i < RB_U; ++i) {
+        const uint32_t v = c0 + i * RB_T + threadIdx.x;
+        w[i] = v < (uint32_t)n ? jw_load(p.jw + b + v) : jw_pack(-1, 0);
+      }
+#pragma unroll
+      for (int i = 0; i < RB_U; ++i) go[i] = (int32_t)(uint32_t)w[i] >= 0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int i = 0; i < RB_U; ++i)
+          if ((int32_t)(uint32_t)w[i] >= 0) x[i] = jw_load(p.jw + (uint32_t)w[i]);
+#pragma unroll
+        for (int i = 0; i < RB_U; ++i)
+          if ((int32_t)(uint32_t)w[i] >= 0)
+            w[i] = jw_pack((int32_t)(uint32_t)x[i], (int32_t)((uint32_t)(w[i] >> 32) + (uint32_t)(x[i] >> 32)));
+      }
+#pragma unroll
+      for (int i = 0; i < RB_U; ++i) {
+        if (go[i]) jw_store(p.jw + b + c0 + i * RB_T + threadIdx.x, w[i]);
+        open |= (int32_t)(uint32_t)w[i] >= 0;
+      }
+    });
+    if (__syncthreads_or(open) && threadIdx.x == 0) atomicOr(&p.ctr[4 + r % 3], 1u);
     if (gtid == 0) p.ctr[4 + (r + 1) % 3] = 0u;  // read two rounds ago, after that round's barrier
     grid.sync();
     if (*(volatile uint32_t*)&p.ctr[4 + r % 3] == 0u) break;  // uniform
@@ -357,32 +359,35 @@ __global__ void __launch_bounds__(RB_T, 5) k_rb(RBParams p) {
       return;
     }
   }
-  // preorder numbers to vertex-major order through a shared-memory tile
-  // (coalesced on both sides); the per-row sums start at zero
+  // preorder numbers and sizes to vertex-major order through a shared-memory
+  // tile (coalesced on both sides); the counts of rows of several segments start
+  // at zero
   for (int64_t v0 = (int64_t)blockIdx.x * RB_TILE; v0 < n; v0 += (int64_t)gridDim.x * RB_TILE) {
     const int32_t nv = (int32_t)std::min<int64_t>(RB_TILE, n - v0);
+    const int wid = threadIdx.x >> 5;
+    // tile -> [v][t]: a lane per tree, a warp per vertex
+    auto flip = [&](int32_t* dst) {
+      __syncthreads();
+      if (lane < Tc)
+        for (int x = wid; x < nv; x += RB_T / 32) dst[VT(lane, v0 + x)] = tile[lane][x];
+      __syncthreads();
+    };
     for (int t = 0; t < Tc; ++t)
-      for (int x = threadIdx.x; x < nv; x += blockDim.x) tile[t][x] = (int32_t)(p.jw[(int64_t)t * n1 + v0 + x] >> 32);
-    __syncthreads();
-    const int64_t k1 = (int64_t)nv * Tc;
-    for (int64_t k = threadIdx.x; k < k1; k += blockDim.x) {
-      const int32_t x = (int32_t)(k / Tc), t = (int32_t)(k - (int64_t)x * Tc);
-      p.tin[v0 * Tc + k] = tile[t][x];
-      if (MODE == 0) {
-        if (p.w) p.sout[v0 * Tc + k] = 0.0;
-        else p.outc[v0 * Tc + k] = 0u;
-      }
+      for (int x = threadIdx.x; x < nv; x += blockDim.x) tile[t][x] = (int32_t)(p.jw[(int64_t)t * n + v0 + x] >> 32);
+    flip(p.tin);
+    for (int t = 0; t < Tc; ++t)
+      for (int x = threadIdx.x; x < nv; x += blockDim.x)
+        tile[t][x] = (int32_t)(1u + (uint32_t)p.word[(int64_t)t * n + v0 + x]);
+    flip(p.size);
+    if (MODE == 0 && !p.w) {
+      const int32_t x = threadIdx.x;  // RB_TILE threads
+      if (x < nv && p.rowptr[v0 + x + 1] - p.rowptr[v0 + x] > RB_SEG)
+        for (int t = 0; t < Tc; ++t) p.outc[VT(t, v0 + x)] = 0u;
     }
-    __syncthreads();
     if (MODE == 1) {  // the tree parents, vertex-major, through the same tile
       for (int t = 0; t < Tc; ++t)
         for (int x = threadIdx.x; x < nv; x += blockDim.x) tile[t][x] = p.parents[(int64_t)t * n + v0 + x];
-      __syncthreads();
-      for (int64_t k = threadIdx.x; k < k1; k += blockDim.x) {
-        const int32_t x = (int32_t)(k / Tc), t = (int32_t)(k - (int64_t)x * Tc);
-        p.pvm[v0 * Tc + k] = tile[t][x];
-      }
-      __syncthreads();
+      flip(p.pvm);
     }
   }
   grid.sync();
@@ -430,71 +435,106 @@ __global__ void __launch_bounds__(RB_T, 5) k_rb(RBParams p) {
   }
 
   // ---- neighbours outside the subtree: a warp per row segment, a lane per
-  // tree (each lane sums its tree's weights in row order; unweighted counts
-  // of the segments of a long row add up exactly) ----
-  // The next segment's record is loaded while the current one is scanned.
-  const int64_t nseg = *p.nseg;
-  int4 nxt = gwarp < nseg ? p.segs[gwarp] : make_int4(0, 0, 0, 0);
-  for (int64_t sg = gwarp; sg < nseg; sg += nwarps) {
-    const int4 sv = nxt;
-    if (sg + nwarps < nseg) nxt = p.segs[sg + nwarps];
-    const int32_t v = sv.x;
-    const int64_t e0 = (int64_t)(((uint64_t)(uint32_t)sv.w << 32) | (uint32_t)sv.z);
-    const int64_t e1 = e0 + sv.y;
-    const bool on = lane < Tc;
-    int32_t lo = 0, hi = 0;
-    if (on) {
-      lo = p.tin[VT(lane, v)];
-      hi = lo + p.size[VT(lane, v)];
-    }
-    double s = 0.0;
-    uint32_t c = 0;
-    // 32 entries at a time: lane j loads entry j, the warp broadcasts them
-    // and each lane tests its own tree, in row order; the preorder numbers of
-    // eight neighbours are loaded before any is tested, so eight loads are in
-    // flight (a neighbour past the row's end reads as inside the subtree)
-    for (int64_t eb = e0; eb < e1; eb += 32) {
-      const int32_t m = (int32_t)std::min<int64_t>(32, e1 - eb);
-      const int32_t uj = lane < m ? __ldg(p.colidx + eb + lane) : 0;
-      const float wj = (p.w && lane < m) ? __ldg(p.w + eb + lane) : 0.f;
-      for (int k0 = 0; k0 < m; k0 += 8) {
-        int32_t tu[8];
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const int32_t u = __shfl_sync(0xffffffffu, uj, (k0 + kk) & 31);
-          tu[kk] = (on && k0 + kk < m) ? p.tin[VT(lane, u)] : lo;
-        }
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const float wk = __shfl_sync(0xffffffffu, wj, (k0 + kk) & 31);
-          if (tu[kk] < lo || tu[kk] >= hi) {
-            if (p.w) s = __dadd_rn(s, (double)wk);
-            else ++c;
-          }
-        }
-      }
-    }
-    if (on) {
-      if (p.w) p.sout[VT(lane, v)] = s;  // weighted rows are one segment
-      else if (c) atomicAdd(&p.outc[VT(lane, v)], c);
-    }
-  }
-  grid.sync();
-
-  // ---- the conditional probabilities, summed over the chunk's trees ----
-  for (int64_t v = gwarp; v < n; v += nwarps) {
+  // tree (each lane sums its tree's weights in row order).  A lane whose tree
+  // has v as a leaf loads nothing: every neighbour is outside.  A row of one
+  // segment ends with its conditional probabilities, summed over the trees;
+  // longer unweighted rows leave counts, which add up exactly.  The next
+  // segment's numbers and entries are loaded while the current one is scanned. ----
+  const bool on = lane < Tc;
+  auto finish = [&](int32_t v, double s, uint32_t c) {  // 1 / (1 + alpha s), fixed point, to acc
     uint64_t q = 0;
-    if (lane < Tc && p.qtab) {
-      q = p.qtab[p.outc[VT(lane, v)]];  // the same FP64 steps, done once per count
-    } else if (lane < Tc) {
-      const double s = p.w ? p.sout[VT(lane, v)] : (double)p.outc[VT(lane, v)];
+    if (on && p.qtab) {
+      q = p.qtab[c];  // the same FP64 steps, done once per count
+    } else if (on) {
       const double a = p.alpha_v ? p.alpha_v[v] : p.alpha;
-      const double val = __ddiv_rn(1.0, __dadd_rn(1.0, __dmul_rn(a, s)));
+      const double val = __ddiv_rn(1.0, __dadd_rn(1.0, __dmul_rn(a, p.w ? s : (double)c)));
       q = (uint64_t)__dadd_rn(__dmul_rn(val, (double)(1ull << RB_FRAC)), 0.5);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     if (lane == 0) atomicAdd((unsigned long long*)&p.acc[v], (unsigned long long)q);
+  };
+  {
+    const int64_t nseg = *p.nseg;
+    const int4 none = make_int4(0, 0, 0, 0);
+    int4 rec = gwarp < nseg ? p.segs[gwarp] : none;                     // next segment
+    int4 rec2 = gwarp + nwarps < nseg ? p.segs[gwarp + nwarps] : none;  // and the one after it
+    int32_t nlo = 0, nsz = 1, nu = 0;
+    float nw = 0.f;
+    auto prefetch = [&]() {  // the numbers and the first 32 entries of rec's row
+      if (on && rec.y > 0) {
+        nlo = p.tin[VT(lane, rec.x)];
+        nsz = p.size[VT(lane, rec.x)];
+      }
+      const int64_t e0 = (int64_t)(((uint64_t)(uint32_t)rec.w << 32) | (uint32_t)rec.z);
+      if (lane < rec.y) {
+        nu = __ldg(p.colidx + e0 + lane);
+        if (p.w) nw = __ldg(p.w + e0 + lane);
+      }
+    };
+    prefetch();
+    for (int64_t sg = gwarp; sg < nseg; sg += nwarps) {
+      const int4 sv = rec;
+      const int32_t lo = nlo, hi = nlo + nsz;
+      const bool look = on && nsz > 1;
+      int32_t uj = nu;
+      float wj = nw;
+      rec = rec2;
+      rec2 = sg + 2 * nwarps < nseg ? p.segs[sg + 2 * nwarps] : none;
+      prefetch();
+      const int32_t v = sv.x;
+      const int64_t e0 = (int64_t)(((uint64_t)(uint32_t)sv.w << 32) | (uint32_t)sv.z);
+      double s = 0.0;
+      uint32_t c = 0;
+      if (!p.w && !__any_sync(0xffffffffu, look)) {
+        c = (uint32_t)sv.y;
+      } else {
+        // 32 entries at a time: lane j loads entry j, the warp broadcasts them
+        // and each lane tests its own tree, in row order; the preorder numbers
+        // of eight neighbours are loaded before any is tested, so eight loads
+        // are in flight (a neighbour past the row's end reads as inside)
+        for (int32_t eb = 0; eb < sv.y; eb += 32) {
+          const int32_t m = min(32, sv.y - eb);
+          if (eb > 0) {
+            uj = lane < m ? __ldg(p.colidx + e0 + eb + lane) : 0;
+            wj = (p.w && lane < m) ? __ldg(p.w + e0 + eb + lane) : 0.f;
+          }
+          for (int k0 = 0; k0 < m; k0 += 8) {
+            int32_t tu[8];
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+              const int32_t u = __shfl_sync(0xffffffffu, uj, (k0 + kk) & 31);
+              tu[kk] = k0 + kk < m ? lo - 1 : lo;
+              if (look && k0 + kk < m) tu[kk] = p.tin[VT(lane, u)];
+            }
+            if (p.w) {
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) {
+                const float wk = __shfl_sync(0xffffffffu, wj, (k0 + kk) & 31);
+                if (tu[kk] < lo || tu[kk] >= hi) s = __dadd_rn(s, (double)wk);
+              }
+            } else {
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) c += (uint32_t)(tu[kk] - lo) >= (uint32_t)(hi - lo) ? 1u : 0u;
+            }
+          }
+        }
+      }
+      if (p.w || p.rowptr[v + 1] - p.rowptr[v] <= RB_SEG) finish(v, s, c);
+      else if (on && c) atomicAdd(&p.outc[VT(lane, v)], c);
+    }
+  }
+  grid.sync();
+
+  // ---- rows of several segments, and empty rows ----
+  for (int64_t v0 = gwarp * 32; v0 < n; v0 += nwarps * 32) {
+    const int64_t d = v0 + lane < n ? p.rowptr[v0 + lane + 1] - p.rowptr[v0 + lane] : 1;
+    for (unsigned left = __ballot_sync(0xffffffffu, d == 0 || (!p.w && d > RB_SEG)); left != 0u; left &= left - 1u) {
+      const int k = __ffs(left) - 1;
+      const int32_t v = (int32_t)v0 + k;
+      const bool counted = __shfl_sync(0xffffffffu, d, k) > 0;
+      finish(v, 0.0, on && counted ? p.outc[VT(lane, v)] : 0u);
+    }
   }
 #undef VT
 }
@@ -563,17 +603,17 @@ static fc_status tree_chunks(fc_graph* g, int mode, int32_t alpha_idx, const int
   const void* kern = mode == 0 ? (const void*)k_rb<0> : (const void*)k_rb<1>;
   FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RB_T, 0));
   const int grid = std::max(1, per_sm) * nsm;  // every CTA resident: required by the grid barriers
-  // trees per chunk: one per lane, 44 bytes of scratch per (tree, vertex)
+  // trees per chunk: one per lane, 28 bytes of scratch per (tree, vertex)
   // within a sixteenth of the device (1 to 16 GB), flat ids below 2^31
   const int64_t budget = std::max<int64_t>(1ll << 30, std::min<int64_t>(16ll << 30, (int64_t)(g->device_bytes / 16)));
-  const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(budget / (44ll * (n + 1)),
+  const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(budget / (28ll * (n + 1)),
                                                              ((int64_t)1 << 31) / ((int64_t)n + 1) - 1));
   const int64_t Tc_max = std::min<int64_t>(std::min<int64_t>(T, RB_TMAX), cap);
-  const size_t N1 = (size_t)Tc_max * (n + 1), N = (size_t)Tc_max * n;
+  const size_t N = (size_t)Tc_max * n;
   const int64_t seg_max = (int64_t)n + g->nnz / RB_SEG + 1;  // bound on the number of segments
   char* ws = nullptr;
-  const size_t bytes = N1 * 4 * 3 + (size_t)grid * 4 + N1 * 8 * 2 + N * 4 * 2 + N * 8 + 32 +
-                       ((size_t)n + 1) * 8 + (size_t)seg_max * 16 + ((size_t)g->max_deg + 1) * 8 + 256 * 16;
+  const size_t bytes = N * 8 * 2 + N * 4 * 3 + 32 + RB_TMAX * 4 + ((size_t)n + 1) * 8 + (size_t)seg_max * 16 +
+                       ((size_t)g->max_deg + 1) * 8 + 256 * 16;
   FC_CK(cudaMallocAsync((void**)&ws, bytes, st));
   auto carve = [&](size_t b) {
     char* r = ws;
@@ -593,18 +633,14 @@ static fc_status tree_chunks(fc_graph* g, int mode, int32_t alpha_idx, const int
   p.root = mode == 1 ? g->root : -1;
   p.bpar = g->bpar;
   p.binv = g->binv;
-  p.cnt = (uint32_t*)carve(N1 * 4);
-  p.word = (unsigned long long*)carve(N1 * 8);
-  p.rsz = (uint32_t*)carve(N1 * 4);
-  p.jw = (unsigned long long*)carve(N1 * 8);
+  p.word = (unsigned long long*)carve(N * 8);
+  p.jw = (unsigned long long*)carve(N * 8);
   p.size = (int32_t*)carve(N * 4);
   p.tin = (int32_t*)carve(N * 4);
-  p.sout = (double*)carve(N * 8);  // the unweighted counts use its first half
-  p.outc = (uint32_t*)p.sout;
-  p.pvm = (int32_t*)p.sout;        // resistance mode: the tree parents, vertex-major
-  p.rsum = (uint32_t*)carve(N1 * 4);
-  p.bsum = (uint32_t*)carve((size_t)grid * 4);
-  p.ctr = (uint32_t*)carve(32);
+  p.outc = (uint32_t*)carve(N * 4);
+  p.pvm = (int32_t*)p.outc;  // resistance mode: the tree parents, vertex-major
+  p.ctr = (uint32_t*)carve(32 + RB_TMAX * 4);
+  p.tsum = p.ctr + 8;
   const bool table = mode == 0 && g->w == nullptr && g->num_graphs == 0;
   uint64_t* qtab = table ? (uint64_t*)carve(((size_t)g->max_deg + 1) * 8) : nullptr;
   p.qtab = qtab;
@@ -636,9 +672,8 @@ static fc_status tree_chunks(fc_graph* g, int mode, int32_t alpha_idx, const int
     const int32_t Tc = (int32_t)std::min<int64_t>(Tc_max, T - t0);
     p.Tc = Tc;
     p.parents = parents + (size_t)t0 * n;
-    FC_CK(cudaMemsetAsync(p.cnt, 0, (size_t)Tc * (n + 1) * 4, st));
-    FC_CK(cudaMemsetAsync(p.word, 0, (size_t)Tc * (n + 1) * 8, st));
-    FC_CK(cudaMemsetAsync(p.ctr, 0, 32, st));
+    FC_CK(cudaMemsetAsync(p.word, 0, (size_t)Tc * n * 8, st));
+    FC_CK(cudaMemsetAsync(p.ctr, 0, 32 + RB_TMAX * 4, st));
     void* args[] = {&p};
     FC_CK(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(RB_T), args, 0, st));
     FC_LAUNCHED();
