@@ -99,9 +99,10 @@ def profiled_traffic(kname, launched):
     summary covers the kernel and launch shape that ran and the kernel source
     is unchanged since that capture (else None)."""
     import hashlib
-    prof = os.path.join(ROOT, "profiles", "k_wilson_edge_ba_n2e20_tau1024.md")
+    pop = kname.startswith("k_pop")
+    prof = os.path.join(ROOT, "profiles", "k_pop_ba_n2e20_tau1024.md" if pop else "k_wilson_edge_ba_n2e20_tau1024.md")
     src = [os.path.join(ROOT, "paper_2101_06192_gb300", "csrc", f)
-           for f in ("fc_wilson_edge.cu", "fc_wilson_common.cuh", "fc_internal.cuh")]
+           for f in ("fc_pop.cu" if pop else "fc_wilson_edge.cu", "fc_wilson_common.cuh", "fc_internal.cuh")]
     try:
         txt = open(prof).read()
         h = hashlib.sha256(b"".join(open(f, "rb").read() for f in src)).hexdigest()[:16]
@@ -951,7 +952,7 @@ def run_electrical(args):
     else:  # the sampler dominates: 20 B per walk step + 8 B per vertex and tree
         smp_bytes = algorithmic_bytes(out["stats"][1], n, tau)
         smp_s = pm[1] / 1000.0
-        roofline = {"bound": "hbm", "kernel": "k_wilson_edge<flags> on G rooted at the hub (+ visit totals)",
+        roofline = {"bound": "hbm", "kernel": "k_pop on G rooted at the hub (+ visit totals)",
                     "achieved": smp_bytes / smp_s / 1e9, "peak": peak, "unit": "GB/s",
                     "frac": smp_bytes / smp_s / 1e9 / peak, "algorithmic_bytes": smp_bytes,
                     "peak_source": peak_kind, "traffic": None}
@@ -1270,7 +1271,7 @@ def main():
     achieved = alg_bytes / samp_s / 1e9
     peak = float(peaks.get("hbm_gbs", 6800.0))
     kname = {2: "k_wilson_edge<flags, {r}>", 3: "k_wilson_edge<smem bitmap, {r}>",
-             4: "k_wilson_edge<global bitmap, {r}>"}.get(
+             4: "k_wilson_edge<global bitmap, {r}>", 5: "k_pop"}.get(
         launched.get("kernel"), "k_wilson<global state, {r}>").format(r=launched.get("regs"))
     traffic = profiled_traffic(kname, launched) if full else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
