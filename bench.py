@@ -1038,7 +1038,7 @@ def run_solve(args):
             "roofline": {"bound": "hbm",
                          "kernel": ("CG inner iteration (k_cg1: edge-tile SpMV + vector phases, one cooperative "
                                     "launch per refinement step)" if args.rhs == 1 else
-                                    "CG inner iteration (k_spmv_pq_il + vector kernels)"),
+                                    "CG inner iteration (k_il_spmv + vector kernels)"),
                          "achieved": results[0]["achieved_gbs"], "peak": peak, "unit": "GB/s",
                          "frac": results[0]["frac"], "traffic": None, "peak_source": peak_kind},
             "config": {"workload": f"fc_solve, {args.rhs} right-hand sides e_v, rel_tol 1e-9, alpha=1",
@@ -1266,7 +1266,10 @@ def main():
     pops = statistics.mean(s_[0] for s_ in stats)
     deps = statistics.mean(s_[1] for s_ in stats)
     alg_bytes = algorithmic_bytes(deps, n, tau)
-    lay_bytes = layout_bytes(deps, pops, n, tau, R_sum if world == 1 else R_sum // world)
+    # the walker kernels' own layout (not the cycle-popping kernel's)
+    lay_bytes = None
+    if launched.get("kernel") != 5:
+        lay_bytes = layout_bytes(deps, pops, n, tau, R_sum if world == 1 else R_sum // world)
     samp_s = statistics.mean(samp_ms) / 1000.0
     achieved = alg_bytes / samp_s / 1e9
     peak = float(peaks.get("hbm_gbs", 6800.0))
@@ -1279,7 +1282,7 @@ def main():
                 "traffic_over_algorithmic": (traffic / alg_bytes) if traffic else None,
                 "algorithmic_bytes": alg_bytes,
                 "algorithmic_bytes_rule": "20 B per walk step + 8 B per vertex and tree",
-                "layout_bytes": lay_bytes, "layout_frac": lay_bytes / samp_s / 1e9 / peak,
+                "layout_bytes": lay_bytes, "layout_frac": lay_bytes / samp_s / 1e9 / peak if lay_bytes else None,
                 "kernel": kname, "launch": launched,
                 "peak_source": peak_kind, "kernel_ms": 1000.0 * samp_s,
                 "departures_per_launch": deps, "pops_per_launch": pops,
