@@ -75,7 +75,8 @@ def autotune(G, tau: int, probe_trees: int | None = None, seed: int = 12345) -> 
     if key in cache:
         apply(G, cache[key])
         return dict(cache[key], cached=True)
-    shipped = _load(_SHIPPED).get(key[:-1] + "0")  # measured with the edge-record kernel
+    # measured with the edge-record kernel (keyed by the graph class alone, kernel 0)
+    shipped = _load(_SHIPPED).get(key[:-1] + "0") if G.kernel_pref == 2 else None
     if shipped is not None:
         apply(G, shipped)
         return dict(shipped, cached="shipped")
