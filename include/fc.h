@@ -88,8 +88,10 @@ fc_status fc_build_augmented(int32_t n, int64_t nnz, const int64_t* rowptr, cons
  * the union of the graphs' G* glued at u*, a spanning tree of it is one tree
  * per graph, and all the per-vertex entry points below apply unchanged with
  * vertex ids of the union, alpha index 0:
- *   fc_sample_usts   samples tau trees of every graph: work items (graph,
- *                    tree) run largest graph first; steps_out is [graph][tree];
+ *   fc_sample_usts   samples tau trees of every graph (the walker kernels take
+ *                    (graph, tree) items, largest graph first; cycle popping
+ *                    advances a tree of every graph together); steps_out is
+ *                    [graph][tree];
  *                    parents is [tree][n]; the random stacks use union vertex
  *                    ids, so results equal those of the union graph.
  *   fc_forest_farness  Eq. 3 and Def. 2 within each graph (its n and trace).
@@ -103,7 +105,9 @@ fc_status fc_build_batch(int32_t num_graphs, const int64_t* vertex_offsets, int6
 /*
  * Per-graph latency of the last fc_sample_usts on a batch graph: for graph i,
  * the time from the first CTA start of the launch to the completion of the
- * graph's last tree, in ms (%globaltimer).  per_graph_ms: host double[G].
+ * graph's last tree, in ms (%globaltimer).  Under cycle popping a tree is
+ * complete when its last cycle is redrawn, or, where parents are wanted, when
+ * they are written.  per_graph_ms: host double[G].
  * Synchronous.
  */
 fc_status fc_batch_latency(fc_graph* g, double* per_graph_ms);

@@ -30,7 +30,8 @@
 //
 // until a walk phase finds no cycle.  No locks and no state to clear; a top
 // that selects u* is final (it is never on a cycle), so R, C and the
-// departures are counted where entries are drawn.
+// departures are counted where entries are drawn.  A tree of a batch's graph is
+// complete when the last of its cycles is redrawn: every redraw stamps it.
 //
 // The CTAs of one cooperative launch form teams with their own barriers; each
 // team takes its own windows, so while one team waits for its longest walk (a
@@ -278,6 +279,8 @@ __device__ void pop_redraw(const PopParams& p, uint32_t* F, uint32_t* K, const u
     }
     F[it] = w | PW_RED | (PW_ACT << par);
     if (p.visits != nullptr) atomicAdd(p.visits + (size_t)a * p.n + v, 1ull);
+    // (any of the graph's stamps of this phase will do: they are moments apart)
+    if (p.item_ns != nullptr) p.item_ns[(size_t)p.gid[v] * p.tau + (size_t)t] = global_ns();
   }
 }
 
@@ -464,6 +467,14 @@ __device__ uint32_t pop_walk(const PopParams& p, const uint32_t* F, const uint32
   return pops;
 }
 
+// completion times of a batch's trees in rows [g0, g0 + rows): now
+__device__ void pop_stamp(const PopParams& p, int64_t g0, int32_t rows, int cta) {
+  const unsigned long long ns = global_ns();
+  const int64_t len = (int64_t)rows * p.num_graphs;
+  for (int64_t i = (int64_t)cta * PK_T + threadIdx.x; i < len; i += (int64_t)p.ctas * PK_T)
+    p.item_ns[(i / rows) * p.tau + g0 + i % rows] = ns;
+}
+
 __device__ __forceinline__ void pop_stats(const PopParams& p, uint32_t pops) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) pops += __shfl_xor_sync(FULL, pops, o);
@@ -494,6 +505,7 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
     pop_draw<WGT>(p, F, g0, rows, cta);
     if (cta == 0 && threadIdx.x == 0) lc[0] = lc[1] = 0u;
     if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
+    if (p.item_ns != nullptr) pop_stamp(p, g0, rows, cta);  // complete unless a cycle is found
     uint32_t cnt = 0;
     for (uint32_t rd = 0;; ++rd) {
       // round rd: its list in L[rd & 1] (every vertex for rd = 0)
@@ -521,12 +533,7 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
         const int64_t r = i / p.n;
         p.parents[g0 * p.n + i] = (int32_t)(F[r * p.ld + (i - r * p.n)] & PW_ID);
       }
-    }
-    if (p.item_ns != nullptr) {
-      const unsigned long long ns = global_ns();
-      const int64_t len = (int64_t)rows * p.num_graphs;
-      for (int64_t i = (int64_t)cta * PK_T + threadIdx.x; i < len; i += (int64_t)p.ctas * PK_T)
-        p.item_ns[(i / rows) * p.tau + g0 + i % rows] = ns;
+      if (p.item_ns != nullptr) pop_stamp(p, g0, rows, cta);  // the parents are part of the trees
     }
     if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;  // the tops are read before they are drawn again
   }
