@@ -252,25 +252,24 @@ extern "C" fc_status fc_group_closeness(fc_graph* g, int32_t alpha_idx, int32_t 
   const int64_t ld = ((int64_t)n1 + 3) & ~(int64_t)3;  // row stride of M: 32-byte aligned rows
   int nsm = 0;
   FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
-  // Omega (n^2), M (n1 x ld), the identity block and the solver's scratch
-  // (FP64 residual, four FP32 vectors and, for 32 or more right-hand sides,
-  // interleaved copies of b and x: about 40 bytes per right-hand side and vertex)
+  // Omega (n^2), M (n1 x ld), the identity block and the solver's scratch, in
   // batches of at most 4096 columns, equal to within the 128 columns of a warp
   // (4099 columns as 4096 + 3 took 32 iterations for the three)
   const int32_t nbat = (n + 4095) / 4096;
   const int32_t nb = std::min<int32_t>(n, ((n + nbat - 1) / nbat + 127) & ~127);
-  const size_t need = (size_t)n * n * 8 + (size_t)n1 * ld * 8 + (size_t)nb * n * (8 + 40);
+  const size_t need = (size_t)n * n * 8 + (size_t)n1 * ld * 8 + (size_t)nb * n * 8 + solve_scratch_bytes(g, nb);
   size_t freeb = 0, totb = 0;
   FC_CK(cudaMemGetInfo(&freeb, &totb));
   if (need > freeb / 10 * 9) {
     set_error("fc_group_closeness: the dense matrices do not fit in device memory");
     return FC_ENOMEM;
   }
+  CallScratch scr(st);
   double *Om = nullptr, *M = nullptr, *B = nullptr, *vec = nullptr;
   int32_t* vp = nullptr;
   uint8_t* chosen = nullptr;
-  FC_CK(cudaMallocAsync((void**)&Om, (size_t)n * n * 8, st));
-  FC_CK(cudaMallocAsync((void**)&B, (size_t)nb * n * 8, st));
+  FC_CK(scr.get(&Om, (size_t)n * n * 8));
+  FC_CK(scr.get(&B, (size_t)nb * n * 8));
   // Omega, column block by column block (column j is also row j: symmetric)
   fc_status r = FC_OK;
   for (int32_t j0 = 0; j0 < n && r == FC_OK; j0 += nb) {
@@ -282,15 +281,12 @@ extern "C" fc_status fc_group_closeness(fc_graph* g, int32_t alpha_idx, int32_t 
     FC_CK(cudaMemsetAsync(X, 0, (size_t)cnt * n * 8, st));
     r = fc_solve(g, alpha_idx, B, X, cnt, rel_tol, 100000, nullptr, stream);
   }
-  FC_CK(cudaFreeAsync(B, st));
-  if (r != FC_OK) {
-    FC_CK(cudaFreeAsync(Om, st));
-    return r;
-  }
-  FC_CK(cudaMallocAsync((void**)&M, (size_t)n1 * ld * 8, st));
-  FC_CK(cudaMallocAsync((void**)&vec, (size_t)3 * ld * 8, st));  // m, gain, diag
-  FC_CK(cudaMallocAsync((void**)&vp, 16, st));
-  FC_CK(cudaMallocAsync((void**)&chosen, (size_t)n1, st));
+  if (r != FC_OK) return r;
+  scr.drop(B);
+  FC_CK(scr.get(&M, (size_t)n1 * ld * 8));
+  FC_CK(scr.get(&vec, (size_t)3 * ld * 8));  // m, gain, diag
+  FC_CK(scr.get(&vp, 16));
+  FC_CK(scr.get(&chosen, (size_t)n1));
   double* m = vec;
   double* gain = vec + ld;
   double* diag = vec + 2 * ld;
@@ -300,7 +296,7 @@ extern "C" fc_status fc_group_closeness(fc_graph* g, int32_t alpha_idx, int32_t 
   const unsigned rb = (unsigned)std::min<int64_t>(n1, (int64_t)nsm * 8);
   k_grp_form<<<rb, GR_T, 0, st>>>(n, ld, Om, vp, M);
   FC_LAUNCHED();
-  FC_CK(cudaFreeAsync(Om, st));
+  scr.drop(Om);
   // gains of the starting inverse; v0's row is zero, so its gain is -1
   k_grp_pass<<<rb, GR_T, 0, st>>>(n, ld, M, m, nullptr, chosen, gain, diag);
   FC_LAUNCHED();
@@ -314,10 +310,7 @@ extern "C" fc_status fc_group_closeness(fc_graph* g, int32_t alpha_idx, int32_t 
     k_grp_trace<<<1, GR_T, 0, st>>>(n, diag, k - 1, farness_out);
     FC_LAUNCHED();
   }
-  FC_CK(cudaFreeAsync(M, st));
-  FC_CK(cudaFreeAsync(vec, st));
-  FC_CK(cudaFreeAsync(vp, st));
-  FC_CK(cudaFreeAsync(chosen, st));
+  scr.release();
   FC_CK(cudaStreamSynchronize(st));
   return FC_OK;
 }

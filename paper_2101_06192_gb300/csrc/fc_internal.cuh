@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -46,6 +47,39 @@ void free_graph_arrays(fc_graph* g, cudaStream_t st);
 
 // Keep freed stream-ordered allocations in the device's default pool.
 void retain_pool(int device);
+
+// Device scratch of one call from the stream-ordered pool; what is still held
+// when the call leaves, by whichever return, is freed on the stream.
+class CallScratch {
+ public:
+  explicit CallScratch(cudaStream_t st) : st_(st) {}
+  CallScratch(const CallScratch&) = delete;
+  CallScratch& operator=(const CallScratch&) = delete;
+  ~CallScratch() { release(); }
+  template <typename T>
+  cudaError_t get(T** p, size_t bytes) {
+    void* q = nullptr;
+    const cudaError_t e = cudaMallocAsync(&q, bytes, st_);
+    if (e == cudaSuccess) held_.push_back(q);
+    *p = (T*)q;
+    return e;
+  }
+  void drop(void* p) {
+    cudaFreeAsync(p, st_);
+    held_.erase(std::find(held_.begin(), held_.end(), p));
+  }
+  void release() {
+    for (void* q : held_) cudaFreeAsync(q, st_);
+    held_.clear();
+  }
+
+ private:
+  cudaStream_t st_;
+  std::vector<void*> held_;
+};
+
+// Upper bound on the device scratch of fc_solve with n_rhs right-hand sides.
+size_t solve_scratch_bytes(const fc_graph* g, int32_t n_rhs);
 
 // Exclusive prefix sum of len uint32 values on `st` (multi-level, temporary
 // memory from the stream-ordered pool).

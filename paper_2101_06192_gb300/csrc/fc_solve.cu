@@ -1349,6 +1349,36 @@ static void il_launch_correct(const ILPlan& pl, int32_t n, int m, const double* 
   note_launch();
 }
 
+// Columns of a solve with n_rhs right-hand sides.  Values per lane: a warp takes
+// up to 64 columns, and 128 in 16-byte accesses from 128 on.  The columns are
+// filled up with zero columns (never active) to a multiple of them (R-MAT 2^16:
+// 33 columns 12.9 ms, 63 17.6 -> 13.4 against one value per lane; 96 columns 19.7
+// with two values, 21.6 with four; filling up to 8 or 16 columns changes less
+// than 5% either way).
+static int il_values(int n_rhs) { return n_rhs >= 128 ? 4 : n_rhs > 32 ? 2 : 1; }
+static int il_columns(int n_rhs) {
+  const int pad = il_values(n_rhs) - 1;
+  return n_rhs + pad <= 65535 ? (n_rhs + pad) & ~pad : n_rhs;
+}
+
+// Bytes of the partial sums of rows of several segments of `len` entries, at
+// most: only rows longer than len have them, fewer than 2 d / len each.
+static size_t il_long_bytes(const fc_graph* g, int len, int m) {
+  return g->max_deg <= len ? 0 : (size_t)(2 * g->nnz / len + 1) * m * sizeof(double);
+}
+
+// Entries per segment: IL_SEG or IL_SEG_PACK, doubled while the partial sums
+// could take more than an FP64 vector block and IL_LONG bytes.  Sparse graphs
+// (mean degree up to len / 2) never are; on a complete graph of n = 20,000 the
+// sums of 4096 columns would take 100 GB.
+constexpr size_t IL_LONG = 256u << 20;
+static int il_seg_len(const fc_graph* g, int m) {
+  int len = m > 16 ? IL_SEG : IL_SEG_PACK;
+  const size_t most = std::max(IL_LONG, (size_t)g->n * m * sizeof(double));
+  while (il_long_bytes(g, len, m) > most) len *= 2;
+  return len;
+}
+
 #define IL_DISPATCH(vw, call4, call2, call1) \
   do {                                       \
     if ((vw) == 4) call4;                    \
@@ -1356,26 +1386,23 @@ static void il_launch_correct(const ILPlan& pl, int32_t n, int m, const double* 
     else call1;                              \
   } while (0)
 
+// FP64 residual and copies of b and x, four FP32 vectors, and what the rows need
+size_t solve_scratch_bytes(const fc_graph* g, int32_t n_rhs) {
+  const int m = il_columns(n_rhs), len = il_seg_len(g, m);
+  const size_t n = (size_t)g->n, lmax = (size_t)(g->nnz / len) + 1;
+  return n * m * 40 + il_long_bytes(g, len, m) + (n + 2 * lmax) * 16 + n * 32 + (16u << 20) + (size_t)m * 64;
+}
+
 }  // namespace fcx
 
 using namespace fcx;
 
-static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, double* x, int32_t n_rhs,
-                            double rel_tol, int32_t max_iter, int32_t* iters_out, cudaStream_t st, bool jacobi,
-                            double sigma = 1.0) {
-  if (g == nullptr || b == nullptr || x == nullptr || n_rhs < 1 || n_rhs > 65535 || alpha_idx < 0 ||
-      alpha_idx >= g->n_alpha || !(rel_tol > 0.0) || max_iter < 1) {
-    set_error("fc_solve: bad argument");
-    return FC_EINVAL;
-  }
+// Scratch of a call of several columns: 40 bytes per column and vertex.
+static fc_status solve_columns(fc_graph* g, int32_t alpha_idx, const double* b, double* x, int32_t n_rhs,
+                               double rel_tol, int32_t max_iter, int32_t* iters_out, cudaStream_t st, bool jacobi,
+                               double sigma) {
   const int32_t n = g->n;
-  // values per lane: a warp takes up to 64 columns, and 128 in 16-byte accesses
-  // from 128 on.  The columns are filled up with zero columns (never active) to a
-  // multiple of them (R-MAT 2^16: 33 columns 12.9 ms, 63 17.6 -> 13.4 against one
-  // value per lane; 96 columns 19.7 with two values, 21.6 with four; filling up
-  // to 8 or 16 columns changes less than 5% either way)
-  const int vw = n_rhs >= 128 ? 4 : n_rhs > 32 ? 2 : 1, pad = vw - 1;
-  const int m = n_rhs + pad <= 65535 ? (n_rhs + pad) & ~pad : n_rhs;
+  const int vw = il_values(n_rhs), m = il_columns(n_rhs);
   const double alpha = g->alphas[alpha_idx];
   const int nb = (n + SV_T - 1) / SV_T;  // blocks of the element-wise kernels
   const size_t nm = (size_t)n * m;
@@ -1386,14 +1413,15 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   const bool il = m >= 2 || !coop;
   ILPlan il32{}, il64{};  // FP32 products and vectors, FP64 residual
   // scratch: FP64 r64, FP32 r/p/q/d, diag32, partials, scalars
+  CallScratch scr(st);
   double* r64 = nullptr;
   float* f32 = nullptr;
   double* part = nullptr;
   double* scal = nullptr;
   // each FP32 vector starts on a 16-byte boundary (four-wide accesses)
   const size_t nmp = (nm + 3) & ~(size_t)3, np4 = ((size_t)n + 3) & ~(size_t)3;
-  FC_CK(cudaMallocAsync((void**)&r64, nm * sizeof(double), st));
-  FC_CK(cudaMallocAsync((void**)&f32, (4 * nmp + 2 * np4) * sizeof(float), st));
+  FC_CK(scr.get(&r64, nm * sizeof(double)));
+  FC_CK(scr.get(&f32, (4 * nmp + 2 * np4) * sizeof(float)));
   // partial sums per column of the column-major kernels: a few thousand blocks in all
   const int nbx = std::max(1, std::min(nb, 2048 / m));
   int npart = nbx;
@@ -1404,11 +1432,11 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   const int gy = (m + 31) / 32;  // column tiles of the transposes
   uint32_t* any = nullptr;       // x differs from zero on entry
   uint32_t h_any = 1;
-  FC_CK(cudaMallocAsync((void**)&any, 4, st));
+  FC_CK(scr.get(&any, 4));
   FC_CK(cudaMemsetAsync(any, 0, 4, st));
   if (il) {
-    FC_CK(cudaMallocAsync((void**)&bi, nm * sizeof(double), st));
-    FC_CK(cudaMallocAsync((void**)&xi, nm * sizeof(double), st));
+    FC_CK(scr.get(&bi, nm * sizeof(double)));
+    FC_CK(scr.get(&xi, nm * sizeof(double)));
     if (m != n_rhs) {
       FC_CK(cudaMemsetAsync(bi, 0, nm * sizeof(double), st));
       FC_CK(cudaMemsetAsync(xi, 0, nm * sizeof(double), st));
@@ -1419,9 +1447,9 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(n_rhs, n, x, n, xi, m, any);
     FC_LAUNCHED();
     // row segments (k_il_seg_count, _fill)
-    const int len = m > 16 ? IL_SEG : IL_SEG_PACK;
+    const int len = il_seg_len(g, m);
     const size_t n1 = (size_t)n + 1, lmax = (size_t)(g->nnz / len) + 1, smax = (size_t)n + lmax;
-    FC_CK(cudaMallocAsync(&seg_mem, (smax + lmax) * 16 + n1 * 4 * 6, st));
+    FC_CK(scr.get(&seg_mem, (smax + lmax) * 16 + n1 * 4 * 6));
     int4* segs = (int4*)seg_mem;
     int4* longs = segs + smax;
     uint32_t* cnt = (uint32_t*)(longs + lmax);
@@ -1440,7 +1468,7 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     FC_CK(cudaMemcpyAsync(h + 2, lidx + n, 4, cudaMemcpyDeviceToHost, st));
     FC_CK(cudaMemcpyAsync(&h_any, any, 4, cudaMemcpyDeviceToHost, st));
     FC_CK(cudaStreamSynchronize(st));
-    FC_CK(cudaMallocAsync(&plong, std::max<size_t>(1, (size_t)h[1] * m * sizeof(double)), st));
+    FC_CK(scr.get(&plong, std::max<size_t>(1, (size_t)h[1] * m * sizeof(double))));
     int nsm = 0;
     FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
     auto plan = [&](int vw) {
@@ -1470,8 +1498,8 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   }
   const double* bv = il ? bi : b;
   double* xv = il ? xi : x;
-  FC_CK(cudaMallocAsync((void**)&part, (size_t)2 * m * npart * sizeof(double) + 4 * m * sizeof(double), st));
-  FC_CK(cudaMallocAsync((void**)&scal, (size_t)8 * m * sizeof(double), st));
+  FC_CK(scr.get(&part, (size_t)2 * m * npart * sizeof(double) + 4 * m * sizeof(double)));
+  FC_CK(scr.get(&scal, (size_t)8 * m * sizeof(double)));
   Inner in;
   in.r = f32;
   in.p = f32 + nmp;
@@ -1504,7 +1532,7 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     // [s32 n4][s64 n4][head64 nt][tail64 nt][head32 nt][tail32 nt][row0 nt][row1 nt][meta nt TL_T][span]
     const size_t nsw = ((size_t)n + 31) / 32;
     const size_t bytes = np4 * 12 + nt * 16 + nt * 8 + nt * 8 + nt * TL_T * 4 + nsw * 4 + 16;
-    FC_CK(cudaMallocAsync(&tile_mem, bytes, st));
+    FC_CK(scr.get(&tile_mem, bytes));
     t32.s = (float*)tile_mem;  // 16-byte aligned: B1 reads it four-wide
     t64.s = (double*)(t32.s + np4);
     t64.head = t64.s + np4;
@@ -1557,7 +1585,7 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     tile_grid = (int)std::max<int64_t>(1, std::min<int64_t>((ntiles + TL_W - 1) / TL_W, (int64_t)8 * nsm));
     FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fold ? k_cg1<true> : k_cg1<false>, SV_T, 0));
     cg1_grid = std::max(1, std::min(per_sm, 8)) * nsm;
-    FC_CK(cudaMallocAsync((void**)&cg1_part, (3 * (size_t)cg1_grid + 1) * sizeof(double), st));
+    FC_CK(scr.get(&cg1_part, (3 * (size_t)cg1_grid + 1) * sizeof(double)));
   }
   std::vector<double> h_rr(m), h_bb(m), h_scal((size_t)8 * m, 0.0), h_in(m);
   int used = 0;
@@ -1679,22 +1707,36 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
     const dim3 tg((unsigned)std::min<int64_t>(gy, 1024), (unsigned)std::min<int64_t>((n + 31) / 32, 1024));
     k_il_transpose<<<tg, dim3(32, 8), 0, st>>>(n, n_rhs, xi, m, x, n, nullptr);
     FC_LAUNCHED();
-    FC_CK(cudaFreeAsync(bi, st));
-    FC_CK(cudaFreeAsync(xi, st));
-    FC_CK(cudaFreeAsync(seg_mem, st));
-    FC_CK(cudaFreeAsync(plong, st));
   }
-  FC_CK(cudaFreeAsync(any, st));
-  FC_CK(cudaFreeAsync(r64, st));
-  FC_CK(cudaFreeAsync(f32, st));
-  FC_CK(cudaFreeAsync(part, st));
-  FC_CK(cudaFreeAsync(scal, st));
-  if (cg1_part) FC_CK(cudaFreeAsync(cg1_part, st));
-  if (tile_mem) FC_CK(cudaFreeAsync(tile_mem, st));
+  scr.release();
   FC_CK(cudaStreamSynchronize(st));
   if (iters_out) *iters_out = used;
   if (result != FC_OK) set_error("fc_solve: max_iter reached before rel_tol");
   return result;
+}
+
+// The columns are independent: where the scratch of all of them does not fit
+// (nothing has been written to x then), they are solved in halves.
+static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, double* x, int32_t n_rhs,
+                            double rel_tol, int32_t max_iter, int32_t* iters_out, cudaStream_t st, bool jacobi,
+                            double sigma = 1.0) {
+  if (g == nullptr || b == nullptr || x == nullptr || n_rhs < 1 || n_rhs > 65535 || alpha_idx < 0 ||
+      alpha_idx >= g->n_alpha || !(rel_tol > 0.0) || max_iter < 1) {
+    set_error("fc_solve: bad argument");
+    return FC_EINVAL;
+  }
+  const fc_status s =
+      solve_columns(g, alpha_idx, b, x, n_rhs, rel_tol, max_iter, iters_out, st, jacobi, sigma);
+  if (s != FC_ENOMEM || n_rhs == 1) return s;
+  (void)cudaGetLastError();  // the refused allocation
+  const int32_t h = n_rhs / 2;
+  int32_t it[2] = {0, 0};
+  const size_t off = (size_t)h * g->n;
+  const fc_status s0 = solve_impl(g, alpha_idx, b, x, h, rel_tol, max_iter, &it[0], st, jacobi, sigma);
+  if (s0 != FC_OK && s0 != FC_ENOCONV) return s0;
+  const fc_status s1 = solve_impl(g, alpha_idx, b + off, x + off, n_rhs - h, rel_tol, max_iter, &it[1], st, jacobi, sigma);
+  if (iters_out) *iters_out = std::max(it[0], it[1]);
+  return s1 != FC_OK ? s1 : s0;
 }
 
 extern "C" fc_status fc_solve(fc_graph* g, int32_t alpha_idx, const double* b, double* x, int32_t n_rhs,
@@ -1714,8 +1756,9 @@ extern "C" fc_status fc_pivot_solve(fc_graph* g, int32_t alpha_idx, double* x, d
   double* part = nullptr;
   const int64_t n1 = (int64_t)n + 1;
   const int nb = (int)((n1 + SV_T - 1) / SV_T);
-  FC_CK(cudaMallocAsync((void**)&rhs, (size_t)n * sizeof(double), st));
-  FC_CK(cudaMallocAsync((void**)&part, (size_t)(nb + 1) * sizeof(double), st));
+  CallScratch scr(st);
+  FC_CK(scr.get(&rhs, (size_t)n * sizeof(double)));
+  FC_CK(scr.get(&part, (size_t)(nb + 1) * sizeof(double)));
   // grounded system: x(u*) = 0, (I + alpha L) x_V = -1/(n+1) 1
   k_fill<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, -1.0 / (double)n1, rhs);
   FC_LAUNCHED();
@@ -1732,8 +1775,7 @@ extern "C" fc_status fc_pivot_solve(fc_graph* g, int32_t alpha_idx, double* x, d
   fcx::note_launch();
   k_shift<<<(unsigned)std::min<int64_t>((n1 + 255) / 256, 152 * 8), 256, 0, st>>>(n1, part + nb, x);
   FC_LAUNCHED();
-  FC_CK(cudaFreeAsync(rhs, st));
-  FC_CK(cudaFreeAsync(part, st));
+  scr.release();
   FC_CK(cudaStreamSynchronize(st));
   return s;
 }
@@ -1766,8 +1808,9 @@ extern "C" fc_status fc_laplacian_solve(fc_graph* g, const double* b, double* x,
   double* rhs = nullptr;
   double* part = nullptr;
   const int nb = std::max(1, std::min((n + SV_T - 1) / SV_T, 2048 / n_rhs));
-  FC_CK(cudaMallocAsync((void**)&rhs, (size_t)n * n_rhs * sizeof(double), st));
-  FC_CK(cudaMallocAsync((void**)&part, (size_t)n_rhs * (nb + 1) * sizeof(double), st));
+  CallScratch scr(st);
+  FC_CK(scr.get(&rhs, (size_t)n * n_rhs * sizeof(double)));
+  FC_CK(scr.get(&part, (size_t)n_rhs * (nb + 1) * sizeof(double)));
   // b projected onto the range of L (the complement of span(1))
   const fc_status sb = sub_col_means(n, n_rhs, b, rhs, part, nb, st);
   if (sb != FC_OK) return sb;
@@ -1777,8 +1820,7 @@ extern "C" fc_status fc_laplacian_solve(fc_graph* g, const double* b, double* x,
     const fc_status sx = sub_col_means(n, n_rhs, x, x, part, nb, st);
     if (sx != FC_OK) return sx;
   }
-  FC_CK(cudaFreeAsync(part, st));
-  FC_CK(cudaFreeAsync(rhs, st));
+  scr.release();
   FC_CK(cudaStreamSynchronize(st));
   return s;
 }
