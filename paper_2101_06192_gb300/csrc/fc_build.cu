@@ -55,6 +55,26 @@ fc_status sampler_scratch(int device, size_t bytes, cudaStream_t st, void** out,
   return FC_OK;
 }
 
+static struct {
+  int64_t graphs;
+  size_t bytes;
+} g_pop[64];
+
+void pop_graphs(int device, int change) {
+  if (device < 0 || device >= 64) return;
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  g_pop[device].graphs += change;
+  if (g_pop[device].graphs == 0) g_pop[device].bytes = 0;
+}
+
+bool pop_sized(int device, size_t bytes, bool capturing) {
+  if (device < 0 || device >= 64) return !capturing;
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  if (capturing) return bytes <= g_pop[device].bytes;
+  g_pop[device].bytes = std::max(g_pop[device].bytes, bytes);
+  return true;
+}
+
 static bool g_pool_set[64] = {};
 void retain_pool(int device) {
   if (device < 0 || device >= 64 || g_pool_set[device]) return;
@@ -657,6 +677,7 @@ fc_status fcx::build_impl(int32_t n, int64_t nnz, const int64_t* rowptr, const i
   }
   BUILD_CK(cudaStreamSynchronize(st));
   g->id_local = nnz > 0 && h_local * 4 > (unsigned long long)nnz;
+  pop_graphs(g->device, 1);
   *out = g;
   return FC_OK;
 }
@@ -772,6 +793,7 @@ extern "C" void fc_destroy(fc_graph* g) {
   cudaDeviceSynchronize();
   free_graph_arrays(g, st);
   cudaStreamSynchronize(st);
+  pop_graphs(g->device, -1);
   delete g;
 }
 

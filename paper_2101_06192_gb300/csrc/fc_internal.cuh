@@ -38,6 +38,13 @@ void note_launch();
 // demand, reused across graphs and calls, released by fc_release_scratch.
 fc_status sampler_scratch(int device, size_t bytes, cudaStream_t st, void** out, bool capturing = false);
 
+// Largest scratch of the cycle-popping calls on a device, which later captured
+// calls of any graph may take; forgotten with the device's last graph.
+// pop_graphs counts the graphs; pop_sized says whether a call of `bytes` may be
+// captured, and records it when it is not.
+void pop_graphs(int device, int change);
+bool pop_sized(int device, size_t bytes, bool capturing);
+
 // Graph construction shared by fc_build_augmented, fc_build_batch and
 // fc_build_rooted (root >= 0: walks on G whose only exit is that vertex).
 fc_status build_impl(int32_t n, int64_t nnz, const int64_t* rowptr, const int32_t* colidx, const float* w,
@@ -256,7 +263,6 @@ struct fc_graph {
   int64_t shape_val[SHAPE_SLOTS][6] = {};
   bool shape_used[SHAPE_SLOTS] = {};
   int32_t shape_next = 0;
-  size_t pop_bytes = 0;        // largest scratch of a cycle-popping call (sizes later captured calls)
   // scratch owned by the graph
   void* ws = nullptr;          // sampler per-tree state
   size_t ws_bytes = 0;

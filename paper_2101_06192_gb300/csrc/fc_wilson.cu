@@ -725,18 +725,18 @@ static fc_status sample_pop(fc_graph* g, uint64_t seed, int64_t tau, int64_t tre
   }
   int optin = 0;
   FC_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
-  // a captured call needs its scratch sized by an uncaptured one, as for the
-  // walker kernels (whose small graphs live in shared memory and need none)
+  // a captured call needs its scratch sized by an uncaptured one of any graph
+  // of the device, as for the walker kernels (whose small graphs live in shared
+  // memory and need none)
   const bool small = smem_bytes(32, batch ? g->max_ng : g->n, true) + 64 <= (size_t)optin;
   PopPlan pl;
   const int64_t total = (int64_t)(batch ? 1 : g->n_alpha) * tau;  // a row of a batch: one tree of every graph
   const fc_status ps = pop_plan(g, total, &pl);
   if (ps != FC_OK) return ps;
-  if (capturing && !small && g->pop_bytes < pl.bytes) {
+  if (!pop_sized(g->device, pl.bytes, capturing) && !small) {
     set_error("fc_sample_usts_async: sampler scratch must be sized by an uncaptured call before stream capture");
     return FC_EINVAL;
   }
-  g->pop_bytes = std::max(g->pop_bytes, pl.bytes);
   StreamScratch scr;  // of this call alone: calls on other streams have their own
   scr.st = st;
   FC_CK(cudaMallocAsync(&scr.ptr, pl.bytes, st));
