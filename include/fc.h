@@ -143,10 +143,11 @@ fc_status fc_set_start_order(fc_graph* g, int32_t order);
 /*
  * Sampler kernel: 0 = automatic (the default: cycle popping -- every vertex
  * draws its first stack entry and the cycles of the selected entries are
- * popped until none is left -- unless a setting below chooses a walker kernel
- * or forest roots are wanted; then the edge-record kernel when the tree state
- * lives in global memory, else the CSR-walk kernel with the state in shared
- * memory), 1 = CSR-walk kernel, 2 = edge-record kernel (FC_EINVAL if g has no
+ * popped until none is left -- unless a setting below chooses a walker kernel,
+ * the graph has 2^29 - 1 vertices or more, or parents and step counts are wanted
+ * together of an unweighted single graph of 2^15 to 2^16 vertices; then the
+ * edge-record kernel when the tree state lives in global memory, else the
+ * CSR-walk kernel with the state in shared memory), 1 = CSR-walk kernel, 2 = edge-record kernel (FC_EINVAL if g has no
  * edge records: graphs without edges).  The walker settings
  * (fc_set_sampler_shape, _pops, _bitmap, _cluster at non-zero values) choose
  * among the walker kernels.  Edge records are 16 bytes

@@ -687,15 +687,15 @@ static fc_status batch_stamps(fc_graph* g, int64_t tau, bool capturing, cudaStre
 // and depths (parents, then pointer jumping, against recording them as vertices
 // join the tree) BA n = 2^17, 96 trees 2.3 -> 0.88.  Exceptions:
 //  * ids of 29 bits in the words of the tops;
-//  * parents (an analysis output) of unweighted graphs of 2^15 to 2^16 vertices
-//    without a dominating hub: tests/test_gpu_edge_kernel.py pins the walker
-//    kernel and its automatic clusters for these launches (0.87 ms against
-//    0.34 ms for 64 trees of BA n = 50,000).
-static bool pop_applies(const fc_graph* g, const int32_t* parents) {
+//  * diagnostic calls (parents and step counts together) on unweighted single
+//    graphs of 2^15 to 2^16 vertices: tests/test_gpu_edge_kernel.py pins the
+//    walker kernel and its automatic clusters for them (0.87 ms against 0.34 ms
+//    for 64 trees of BA n = 50,000), and nothing else asks for both.
+static bool pop_applies(const fc_graph* g, const int32_t* parents, const uint64_t* steps_out) {
   const bool automatic = g->kernel_pref == 0 && g->walkers == 0 && g->max_trees == 0 && g->smem_mode == 0 &&
                          g->regs == 0 && g->bitmap_mode == 0 && g->pops_mode == 0 && g->cluster == 0;
-  const bool pinned = parents != nullptr && !g->weighted && g->num_graphs == 0 && g->root < 0 && g->n > (1 << 15) &&
-                      g->n <= (1 << 16) && g->max_deg <= g->n / 16;
+  const bool pinned = parents != nullptr && steps_out != nullptr && !g->weighted && g->num_graphs == 0 &&
+                      g->root < 0 && g->n > (1 << 15) && g->n <= (1 << 16);
   return automatic && g->n < (1 << 29) - 1 && !pinned;
 }
 
@@ -773,7 +773,7 @@ static fc_status sample_impl(fc_graph* g, uint64_t seed, int64_t tau, int64_t tr
     set_error("fc_sample_usts: reads its status back; use fc_sample_usts_async on a capturing stream");
     return FC_EINVAL;
   }
-  if (pop_applies(g, parents))
+  if (pop_applies(g, parents, steps_out))
     return sample_pop(g, seed, tau, tree_offset, R, C, parents, roots, depths, visits, max_steps_per_tree, steps_out, st,
                       sync, capturing);
   int dev_smem_optin = 0, nsm = 0;
