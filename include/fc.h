@@ -654,9 +654,12 @@ fc_status fc_sampler_stats(fc_graph* g, uint64_t* pops, uint64_t* departures);
 uint64_t fc_launch_count(void);
 
 /*
- * fc_sample_usts keeps its per-tree state in one process-wide device buffer
- * per GPU, grown on demand and reused by every graph.  This frees those
- * buffers (synchronises the device).  Graphs stay valid.
+ * The walker kernels of fc_sample_usts keep their per-tree state in one
+ * process-wide device buffer per GPU, grown on demand and reused by every
+ * graph; cycle popping and the other entry points take scratch from the
+ * device's default memory pool, where it stays when a call is done.  This frees
+ * those buffers and gives the pools' unused memory back (synchronises the
+ * devices).  Graphs stay valid.
  */
 fc_status fc_release_scratch(void);
 

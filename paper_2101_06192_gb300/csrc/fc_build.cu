@@ -462,6 +462,22 @@ extern "C" fc_status fc_release_scratch(void) {
       sc.bytes = 0;
     }
   }
+  // the cycle-popping sampler's scratch is a stream-ordered allocation of each
+  // call: once freed it stays in the device's pool (retain_pool)
+  int cur = 0;
+  FC_CK(cudaGetDevice(&cur));
+  cudaError_t e = cudaSuccess;
+  for (int d = 0; d < 64 && e == cudaSuccess; ++d) {
+    if (!g_pool_set[d]) continue;
+    cudaMemPool_t pool;
+    e = cudaSetDevice(d);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaDeviceGetDefaultMemPool(&pool, d);
+    if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
+  }
+  const cudaError_t back = cudaSetDevice(cur);
+  if (e != cudaSuccess || back != cudaSuccess)
+    return cuda_fail(e != cudaSuccess ? e : back, "fc_release_scratch: memory pool");
   return FC_OK;
 }
 
