@@ -208,7 +208,8 @@ int32_t fc_sampler_last_cluster(const fc_graph* g);
  * owner has already moved on (its path joined the tree or was released).
  * out: host uint64[count], count >= 10.
  * The counters are compiled in only when the library is built with
- * FC_WILSON_COUNTERS=1 (they cost registers); otherwise they read 0.
+ * FC_WILSON_COUNTERS=1 (they cost registers); otherwise, and after a call by
+ * cycle popping, they read 0.
  * Synchronous.
  */
 fc_status fc_sampler_counters(fc_graph* g, uint64_t* out, int32_t count);

@@ -544,6 +544,7 @@ __global__ void k_pop_begin(unsigned long long* t0_ns, unsigned long long* stats
   if (t0_ns) *t0_ns = global_ns();
   stats[0] = 0;
   stats[1] = departures;
+  for (int i = 0; i < N_CNT; ++i) stats[2 + i] = 0;  // the walkers' counters
 }
 
 }  // namespace
