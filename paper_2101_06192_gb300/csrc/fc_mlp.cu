@@ -15,7 +15,7 @@
 // and the output layer N = 1, so these are per-vertex dot products on the
 // CUDA cores, bound by issue slots: 5 FMAs, a maximum and the weights' loads per
 // vertex and hidden unit, against a 16-byte feature row per vertex.  So a thread
-// of the forward pass takes eight vertices per load of a unit's weights, and a
+// of the forward pass takes up to eight vertices per load of a unit's weights, and a
 // lane of the gradient pass four units per load of a vertex's features.
 // Measured on GB300 (whole calls, against one vertex and one unit): forward pass
 // n = 2^22 190 -> 139 us; loss and gradient n = 2^22 475 -> 397, 2^18 53 -> 42.
@@ -199,25 +199,26 @@ __device__ __forceinline__ float mlp_g(float z, const uint4& ri) {
   return p + (1.0f - p) * s;
 }
 
-constexpr int MLP_NV = 8;  // vertices per thread of the forward pass
+// NV vertices per thread
+template <int NV>
 __global__ void __launch_bounds__(MLP_T) k_mlp_forward(int32_t n, const float4* __restrict__ X,
                                                        const uint4* __restrict__ rinfo,
                                                        const float* __restrict__ params, float* __restrict__ gout) {
   __shared__ Unit su[HID];
   load_params(params, su);
   const float b2 = bf16r(params[OFF_B2]);
-  const int64_t step = MLP_NV * MLP_T;
+  const int64_t step = NV * MLP_T;
   for (int64_t base = blockIdx.x * step; base < n; base += gridDim.x * step) {
-    float4 x[MLP_NV];
-    float z[MLP_NV];
+    float4 x[NV];
+    float z[NV];
 #pragma unroll
-    for (int i = 0; i < MLP_NV; ++i) {
+    for (int i = 0; i < NV; ++i) {
       const int64_t v = base + i * MLP_T + threadIdx.x;
       x[i] = v < n ? X[v] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    mlp_z<MLP_NV>(su, b2, x, z);
+    mlp_z<NV>(su, b2, x, z);
 #pragma unroll
-    for (int i = 0; i < MLP_NV; ++i) {
+    for (int i = 0; i < NV; ++i) {
       const int64_t v = base + i * MLP_T + threadIdx.x;
       if (v < n) gout[v] = mlp_g(z[i], rinfo[v]);
     }
@@ -407,6 +408,12 @@ __global__ void k_adam(int32_t count, float* __restrict__ params, const float* _
   params[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
+// Vertices per thread, at most `most`: two blocks per SM at least.
+static int mlp_vertices(int32_t n, int most) {
+  while (most > 1 && n < (int64_t)152 * 2 * most * MLP_T) most /= 2;
+  return most;
+}
+
 // Blocks for n vertices in tiles of `tile`: at most eight per SM, with equal
 // numbers of tiles.
 static int mlp_blocks(int32_t n, int tile) {
@@ -452,8 +459,12 @@ extern "C" fc_status fc_mlp_forward(fc_graph* g, int32_t alpha_idx, const float*
     return FC_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  k_mlp_forward<<<mlp_blocks(g->n, MLP_NV * MLP_T), MLP_T, 0, st>>>(g->n, (const float4*)X, g->rowinfo + (size_t)alpha_idx * g->n,
-                                                    params, g_out);
+  // vertices per thread: the most that still gives every SM two blocks, as for
+  // the gradient (a thread's vertices share its loads, but run one after another)
+  const int nv = mlp_vertices(g->n, 8);
+  (nv == 8 ? k_mlp_forward<8> : nv == 4 ? k_mlp_forward<4> : nv == 2 ? k_mlp_forward<2> : k_mlp_forward<1>)
+      <<<mlp_blocks(g->n, nv * MLP_T), MLP_T, 0, st>>>(g->n, (const float4*)X, g->rowinfo + (size_t)alpha_idx * g->n,
+                                                       params, g_out);
   FC_LAUNCHED();
   return FC_OK;
 }
@@ -470,8 +481,7 @@ extern "C" fc_status fc_mlp_loss_grad_acc(fc_graph* g, int32_t alpha_idx, const 
   // vertices per thread: the most that still gives every SM two blocks (GB300,
   // whole calls with 1, 2, 4 vertices: n = 2^16 24, 27, - us; 2^17 37, 29, 34;
   // 2^18 54, 45, 42; 2^22 -, 425, 397)
-  int nv = 4;
-  while (nv > 1 && g->n < (int64_t)152 * 2 * nv * MLP_T) nv /= 2;
+  const int nv = mlp_vertices(g->n, 4);
   const int nb = mlp_blocks(g->n, nv * MLP_T);
   float* gpart = nullptr;
   double* lpart = nullptr;
