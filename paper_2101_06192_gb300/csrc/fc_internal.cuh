@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -263,6 +264,7 @@ struct fc_graph {
   int64_t shape_val[SHAPE_SLOTS][6] = {};
   bool shape_used[SHAPE_SLOTS] = {};
   int32_t shape_next = 0;
+  mutable std::atomic<int> pop_per_sm{0};  // resident CTAs per SM of the cycle-popping kernel (0: not asked yet)
   // scratch owned by the graph
   void* ws = nullptr;          // sampler per-tree state
   size_t ws_bytes = 0;

@@ -110,10 +110,21 @@ __device__ __forceinline__ uint32_t ld_top(const uint32_t* a) {
 
 // Barrier of a team (all CTAs of the launch are resident).  Returns true when
 // the launch is to be left: the last CTA to arrive reads the error word for
-// all of them, so they leave together.
+// all of them, so they leave together.  A team of one CTA looks at it every 16th
+// time only (n = 2, three alphas x 50 trees, some 200 rounds each: 451
+// -> 279 us a call, the walker kernels 342).
 __device__ __forceinline__ bool team_sync(uint32_t* ctl, int ctas, uint32_t& gen, const uint32_t* err) {
   __shared__ uint32_t sh_abort;
+  if (ctas == 1 && (++gen & 15u) != 0u) {
+    __syncthreads();
+    return false;
+  }
   __syncthreads();
+  if (ctas == 1) {
+    if (threadIdx.x == 0) sh_abort = *(volatile const uint32_t*)err;
+    __syncthreads();
+    return sh_abort != 0u;
+  }
   if (threadIdx.x == 0) {
     ++gen;
     uint32_t old, g = 0;
@@ -540,7 +551,15 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
   pop_stats(p, pops);
 }
 
-__global__ void k_pop_begin(unsigned long long* t0_ns, unsigned long long* stats, unsigned long long departures) {
+// What a call starts from, in one launch: a call on a tiny graph is launches.
+// n = 3, 1000 trees on GB300, whole calls: 132 us with two clears, a cooperative
+// launch and a full barrier per phase, 102 now (the walker kernels: 112).
+// (ctl: the barriers of teams of several CTAs)
+__global__ void k_pop_begin(unsigned long long* t0_ns, unsigned long long* stats, unsigned long long departures,
+                            uint32_t* err, uint32_t* ctl, int words) {
+  for (int i = threadIdx.x; i < words; i += blockDim.x) ctl[i] = 0u;
+  if (threadIdx.x != 0) return;
+  if (err) *err = 0u;
   if (t0_ns) *t0_ns = global_ns();
   stats[0] = 0;
   stats[1] = departures;
@@ -569,10 +588,13 @@ static const void* pop_fn(const fc_graph* g) {
 }
 
 fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* pl) {
-  int nsm = 0, per_sm = 0, coop = 0;
+  int nsm = 0, coop = 0, per_sm = g->pop_per_sm.load(std::memory_order_relaxed);
   FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
   FC_CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device));
-  FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pop_fn(g), PK_T, 0));
+  if (per_sm == 0) {  // of the kernel and the device alone
+    FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pop_fn(g), PK_T, 0));
+    g->pop_per_sm.store(per_sm, std::memory_order_relaxed);
+  }
   if (!coop || per_sm < 1) {
     set_error("fc_sample_usts: the device does not support cooperative launches");
     return FC_ECUDA;
@@ -593,7 +615,7 @@ fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* pl) {
   return FC_OK;
 }
 
-fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& pl, void* ws, cudaStream_t st) {
+fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& pl, void* ws, bool reset_err, cudaStream_t st) {
   PopParams p;
   p.n = g->n;
   p.nnz = g->nnz;
@@ -634,11 +656,14 @@ fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& pl, void* ws,
   p.err = w.err;
   p.stats = w.stats;
   p.max_iters = w.max_iters;
-  FC_CK(cudaMemsetAsync(p.ctl, 0, (size_t)pl.teams * 128, st));
-  k_pop_begin<<<1, 1, 0, st>>>(w.t0_ns, w.stats, (unsigned long long)g->n * (unsigned long long)p.total);
+  k_pop_begin<<<1, 512, 0, st>>>(w.t0_ns, w.stats, (unsigned long long)g->n * (unsigned long long)p.total,
+                                 reset_err ? w.err : nullptr, p.ctl, pl.ctas == 1 ? 0 : pl.teams * 32);
   FC_LAUNCHED();
   void* args[] = {&p};
-  FC_CK(cudaLaunchCooperativeKernel(pop_fn(g), dim3((unsigned)(pl.teams * pl.ctas)), dim3(PK_T), args, 0, st));
+  const dim3 grid((unsigned)(pl.teams * pl.ctas));
+  // teams of one CTA wait for no other: no cooperative launch
+  FC_CK(pl.ctas == 1 ? cudaLaunchKernel(pop_fn(g), grid, dim3(PK_T), args, 0, st)
+                     : cudaLaunchCooperativeKernel(pop_fn(g), grid, dim3(PK_T), args, 0, st));
   FC_LAUNCHED();
   g->last_W = PK_T;
   g->last_regs = 64;

@@ -723,29 +723,29 @@ static fc_status sample_pop(fc_graph* g, uint64_t seed, int64_t tau, int64_t tre
     p.item_ns = g->item_ns;
     p.t0_ns = g->t0_ns;
   }
-  int optin = 0;
-  FC_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
-  // a captured call needs its scratch sized by an uncaptured one of any graph
-  // of the device, as for the walker kernels (whose small graphs live in shared
-  // memory and need none)
-  const bool small = smem_bytes(32, batch ? g->max_ng : g->n, true) + 64 <= (size_t)optin;
   PopPlan pl;
   const int64_t total = (int64_t)(batch ? 1 : g->n_alpha) * tau;  // a row of a batch: one tree of every graph
   const fc_status ps = pop_plan(g, total, &pl);
   if (ps != FC_OK) return ps;
-  if (!pop_sized(g->device, pl.bytes, capturing) && !small) {
-    set_error("fc_sample_usts_async: sampler scratch must be sized by an uncaptured call before stream capture");
-    return FC_EINVAL;
+  // a captured call needs its scratch sized by an uncaptured one of any graph
+  // of the device, as for the walker kernels (whose small graphs live in shared
+  // memory and need none)
+  if (!pop_sized(g->device, pl.bytes, capturing)) {
+    int optin = 0;
+    FC_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device));
+    if (smem_bytes(32, batch ? g->max_ng : g->n, true) + 64 > (size_t)optin) {
+      set_error("fc_sample_usts_async: sampler scratch must be sized by an uncaptured call before stream capture");
+      return FC_EINVAL;
+    }
   }
   StreamScratch scr;  // of this call alone: calls on other streams have their own
   scr.st = st;
   FC_CK(cudaMallocAsync(&scr.ptr, pl.bytes, st));
-  if (sync) FC_CK(cudaMemsetAsync(g->d_err, 0, sizeof(uint32_t), st));
   // forest roots and depths: by pointer jumping over the parents, in place
   // when they are not asked for
   const bool want_roots = roots != nullptr || depths != nullptr;
   if (want_roots && parents == nullptr) p.parents = roots != nullptr ? roots : depths;
-  const fc_status s = pop_sample(g, p, pl, scr.ptr, st);
+  const fc_status s = pop_sample(g, p, pl, scr.ptr, sync, st);
   if (s != FC_OK || !sync) return s;
   uint32_t herr = 0;
   FC_CK(cudaMemcpyAsync(&herr, g->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));

@@ -171,6 +171,7 @@ struct PopPlan {
   size_t bytes;     // scratch
 };
 fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* plan);
-fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& plan, void* ws, cudaStream_t st);
+// reset_err: clear the error word first.
+fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& plan, void* ws, bool reset_err, cudaStream_t st);
 
 }  // namespace fcx
