@@ -90,7 +90,9 @@ fc_status cuda_fail(cudaError_t e, const char* what) {
   char buf[512];
   snprintf(buf, sizeof(buf), "%s: %s", what, cudaGetErrorString(e));
   set_error(buf);
-  return e == cudaErrorMemoryAllocation ? FC_ENOMEM : FC_ECUDA;
+  if (e != cudaErrorMemoryAllocation) return FC_ECUDA;
+  (void)cudaGetLastError();  // a refused allocation leaves the context whole: not the next launch's error
+  return FC_ENOMEM;
 }
 
 // ---------------------------------------------------------------------------

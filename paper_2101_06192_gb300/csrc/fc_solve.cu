@@ -1774,7 +1774,6 @@ static fc_status solve_impl(fc_graph* g, int32_t alpha_idx, const double* b, dou
   const fc_status s =
       solve_columns(g, alpha_idx, b, x, n_rhs, rel_tol, max_iter, iters_out, st, jacobi, sigma);
   if (s != FC_ENOMEM || n_rhs == 1) return s;
-  (void)cudaGetLastError();  // the refused allocation
   const int32_t h = n_rhs / 2;
   int32_t it[2] = {0, 0};
   const size_t off = (size_t)h * g->n;

@@ -126,3 +126,16 @@ def test_refused_allocation_leaves_nothing_behind():
         assert bool((x == 0.25).all())
         x, _ = G.solve(b, rel_tol=1e-10)
     np.testing.assert_allclose(x.sum(1).cpu().numpy(), 1.0, atol=1e-7)  # 1^T (I + L)^-1 = 1^T
+
+
+def test_refused_allocation_is_the_error_of_its_own_call():
+    """One column, refused; the next call of the thread launches and returns."""
+    g = synth.torus(2048, 1024)
+    with fc.Graph.from_csr(g, [1.0]) as G:
+        b = _unit_columns(g.n, 1)
+        with _own_pool(32 * MB):
+            with pytest.raises(fc.FcError) as e:
+                G.solve(b)
+            assert e.value.status == fc.FC_ENOMEM
+            with fc.Graph.from_csr(synth.path(10), [1.0]) as P:
+                assert P.sample(1, 4)["R"].numel() == 10
