@@ -106,8 +106,8 @@ fc_status fc_build_batch(int32_t num_graphs, const int64_t* vertex_offsets, int6
  * Per-graph latency of the last fc_sample_usts on a batch graph: for graph i,
  * the time from the first CTA start of the launch to the completion of the
  * graph's last tree, in ms (%globaltimer).  Under cycle popping a tree is
- * complete when its last cycle is redrawn, or, where parents are wanted, when
- * they are written.  per_graph_ms: host double[G].
+ * complete when its last cycle is found, which is popped in the same round, or,
+ * where parents are wanted, when they are written.  per_graph_ms: host double[G].
  * Synchronous.
  */
 fc_status fc_batch_latency(fc_graph* g, double* per_graph_ms);

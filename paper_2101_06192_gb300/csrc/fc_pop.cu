@@ -31,7 +31,7 @@
 // until a walk phase finds no cycle.  No locks and no state to clear; a top
 // that selects u* is final (it is never on a cycle), so R, C and the
 // departures are counted where entries are drawn.  A tree of a batch's graph is
-// complete when the last of its cycles is redrawn: every redraw stamps it.
+// complete when its last cycle is listed for its redraw: every listing stamps it.
 //
 // The CTAs of one cooperative launch form teams with their own barriers; each
 // team takes its own windows, so while one team waits for its longest walk (a
@@ -101,7 +101,8 @@ constexpr uint32_t GEN_ABORT = 0x80000000u;
 constexpr uint32_t POP_SPIN = 1u << 23;  // polls of a barrier before it gives up
 
 // Tops within a walk phase, where nothing writes them: cached in L1 (the
-// barrier's acquire drops lines of the phases before).
+// barrier's acquire drops lines of the phases before; a team of one CTA writes
+// its tops from the same SM, and the block's barrier orders its threads).
 __device__ __forceinline__ uint32_t ld_top(const uint32_t* a) {
   uint32_t v;
   asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
@@ -113,14 +114,15 @@ __device__ __forceinline__ uint32_t ld_top(const uint32_t* a) {
 // all of them, so they leave together.  A team of one CTA looks at it every 16th
 // time only (n = 2, three alphas x 50 trees, some 200 rounds each: 451
 // -> 279 us a call, the walker kernels 342).
+template <bool ONE>
 __device__ __forceinline__ bool team_sync(uint32_t* ctl, int ctas, uint32_t& gen, const uint32_t* err) {
   __shared__ uint32_t sh_abort;
-  if (ctas == 1 && (++gen & 15u) != 0u) {
+  if (ONE && (++gen & 15u) != 0u) {
     __syncthreads();
     return false;
   }
   __syncthreads();
-  if (ctas == 1) {
+  if (ONE) {
     if (threadIdx.x == 0) sh_abort = *(volatile const uint32_t*)err;
     __syncthreads();
     return sh_abort != 0u;
@@ -184,7 +186,7 @@ __device__ __forceinline__ uint32_t slot_search(const uint64_t* b, uint32_t d, u
 // draw: entry 0 of every vertex in rows [g0, g0 + rows); a thread per vertex,
 // the rows in a loop (row info, and a short row's thresholds, in registers;
 // the targets of the row stay in L1).
-template <bool WGT>
+template <bool WGT, bool BAT>
 __device__ void pop_draw(const PopParams& p, uint32_t* F, int64_t g0, int32_t rows, int cta) {
   const int32_t nv = (p.n + PK_T - 1) / PK_T;
   // rows per task: as many as leave two tasks per CTA
@@ -202,7 +204,7 @@ __device__ void pop_draw(const PopParams& p, uint32_t* F, int64_t g0, int32_t ro
     row_of(p, g0 + r, &a, &t);
     int32_t gi = 0, nl = p.n;
     bool lead = v == 0 && p.steps != nullptr;
-    if (p.num_graphs > 0 && p.steps != nullptr) {
+    if (BAT && p.steps != nullptr) {
       gi = p.gid[v];
       lead = p.voff[gi] == v;
       nl = (int32_t)(p.voff[gi + 1] - v);
@@ -250,7 +252,7 @@ __device__ void pop_draw(const PopParams& p, uint32_t* F, int64_t g0, int32_t ro
       }
       if (p.visits != nullptr) atomicAdd(p.visits + (size_t)a * p.n + v, (unsigned long long)(r - rb));
       if (lead) {
-        unsigned long long* s = p.steps + (p.num_graphs > 0 ? (size_t)gi : (size_t)a) * p.tau + (size_t)t;
+        unsigned long long* s = p.steps + (BAT ? (size_t)gi : (size_t)a) * p.tau + (size_t)t;
         for (int32_t q = rb; q < r; ++q) s[q - rb] = (unsigned long long)nl;
       }
       ++a;
@@ -261,7 +263,7 @@ __device__ void pop_draw(const PopParams& p, uint32_t* F, int64_t g0, int32_t ro
 
 // redraw: the next stack entry of every listed vertex; the last round's ACT
 // flags are cleared (a vertex in both lists ends with the new word either way)
-template <bool WGT>
+template <bool WGT, bool BAT>
 __device__ void pop_redraw(const PopParams& p, uint32_t* F, uint32_t* K, const uint32_t* list, uint32_t cnt,
                            const uint32_t* old, uint32_t oldcnt, int par, int64_t g0, int cta) {
   const uint32_t stride = (uint32_t)p.ctas * PK_T;
@@ -290,23 +292,25 @@ __device__ void pop_redraw(const PopParams& p, uint32_t* F, uint32_t* K, const u
     }
     F[it] = w | PW_RED | (PW_ACT << par);
     if (p.visits != nullptr) atomicAdd(p.visits + (size_t)a * p.n + v, 1ull);
-    // (any of the graph's stamps of this phase will do: they are moments apart)
-    if (p.item_ns != nullptr) p.item_ns[(size_t)p.gid[v] * p.tau + (size_t)t] = global_ns();
   }
 }
 
 // The vertices of the cycles whose finders are listed in own[0, cnt), a lane
 // per cycle: round once for the lengths, once more to append the vertices (the
 // walk that found the cycle left its tops in L1).
+template <bool BAT>
 __device__ uint32_t pop_list_cycles(const PopParams& p, const uint32_t* F, const uint32_t* own, int cnt, uint32_t* out,
                                     uint32_t* outcnt, int64_t g0) {
   const int lane = threadIdx.x & 31;
   uint32_t rb = 0, v = 0, len = 0, row = 0;
+  int32_t gi = 0;
+  const unsigned long long ns = BAT ? global_ns() : 0ull;
   if (lane < cnt) {
     const uint32_t it = own[lane];
     row = row_of_item(p, it);
     rb = row * p.ld;
     v = it - rb;
+    if (BAT) gi = __ldg(p.gid + v);  // needed at the end
     uint32_t x = v;
     do {
       x = ld_top(F + (rb + x)) & PW_ID;
@@ -334,9 +338,14 @@ __device__ uint32_t pop_list_cycles(const PopParams& p, const uint32_t* F, const
       int32_t a;
       int64_t t;
       row_of(p, g0 + row, &a, &t);
-      atomicAdd(p.steps + (p.num_graphs > 0 ? (size_t)p.gid[v] : (size_t)a) * p.tau + (size_t)t,
+      atomicAdd(p.steps + (BAT ? (size_t)gi : (size_t)a) * p.tau + (size_t)t,
                 (unsigned long long)len);
     }
+    // the tree's completion time, unless it has a cycle in a later round too (any
+    // of the stamps that it gets in this phase will do: they are moments apart).
+    // 256 uneven graphs, 64 trees on GB300: a stamp per cycle with the graph's
+    // number loaded ahead costs 1.3% of a call, one per redrawn vertex 3 to 5%
+    if (BAT) p.item_ns[(size_t)gi * p.tau + (size_t)(g0 + row)] = ns;
   }
   __syncwarp();
   return len;
@@ -350,7 +359,7 @@ __device__ uint32_t pop_list_cycles(const PopParams& p, const uint32_t* F, const
 // dependent loads, so every lane is kept on a walk: candidates wait in a ring
 // in shared memory, and the words of the next unit (PK_CHUNK vertices of a
 // row, or 32 listed vertices) are loaded while the lanes walk.
-template <bool FIRST>
+template <bool FIRST, bool BAT>
 __device__ uint32_t pop_walk(const PopParams& p, const uint32_t* F, const uint32_t* list, uint32_t cnt, int par,
                              uint32_t* out, uint32_t* outcnt, int64_t g0, int32_t rows, int cta, uint2* q,
                              uint32_t* own) {
@@ -467,13 +476,13 @@ __device__ uint32_t pop_walk(const PopParams& p, const uint32_t* F, const uint32
       no += __popc(m);
       __syncwarp();
       if (no >= 32) {
-        pops += pop_list_cycles(p, F, own + (no - 32), 32, out, outcnt, g0);
+        pops += pop_list_cycles<BAT>(p, F, own + (no - 32), 32, out, outcnt, g0);
         no -= 32;
         __syncwarp();
       }
     }
   }
-  if (no) pops += pop_list_cycles(p, F, own, no, out, outcnt, g0);
+  if (no) pops += pop_list_cycles<BAT>(p, F, own, no, out, outcnt, g0);
   __syncwarp();
   return pops;
 }
@@ -495,7 +504,10 @@ __device__ __forceinline__ void pop_stats(const PopParams& p, uint32_t pops) {
   }
 }
 
-template <bool WGT>
+// BAT: a batch (steps and completion times per graph); ONE: teams of one CTA.
+// Templates, because the kernel is at its 64 registers (BA n = 2^20 from CSR, 1024
+// trees, whole calls: 24.87 ms with both decided at run time, 24.27 so).
+template <bool WGT, bool BAT, bool ONE>
 __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
   __shared__ uint2 sh_q[PK_W][PK_RING];
   __shared__ uint32_t sh_e[PK_W][PK_OWN];
@@ -513,10 +525,10 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
   for (int64_t win = team; win < windows; win += p.teams) {
     const int64_t g0 = win * p.wrows;
     const int32_t rows = (int32_t)min((int64_t)p.wrows, p.total - g0);
-    pop_draw<WGT>(p, F, g0, rows, cta);
+    pop_draw<WGT, BAT>(p, F, g0, rows, cta);
     if (cta == 0 && threadIdx.x == 0) lc[0] = lc[1] = 0u;
-    if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
-    if (p.item_ns != nullptr) pop_stamp(p, g0, rows, cta);  // complete unless a cycle is found
+    if ((quit = team_sync<ONE>(ctl, p.ctas, gen, p.err))) break;
+    if (BAT) pop_stamp(p, g0, rows, cta);  // complete unless a cycle is found
     uint32_t cnt = 0;
     for (uint32_t rd = 0;; ++rd) {
       // round rd: its list in L[rd & 1] (every vertex for rd = 0)
@@ -526,16 +538,16 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
         lc[(rd + 2) % 3] = 0u;  // last read two barriers ago
         if (rd > p.max_iters) atomicOr(p.err, ERR_TIMEOUT);
       }
-      if (rd == 0) pops += pop_walk<true>(p, F, cur, 0u, 0, nxt, lc + 1, g0, rows, cta, sh_q[wid], sh_e[wid]);
+      if (rd == 0) pops += pop_walk<true, BAT>(p, F, cur, 0u, 0, nxt, lc + 1, g0, rows, cta, sh_q[wid], sh_e[wid]);
       else
-        pops += pop_walk<false>(p, F, cur, cnt, (int)(rd & 1u), nxt, lc + (rd + 1) % 3, g0, rows, cta, sh_q[wid],
+        pops += pop_walk<false, BAT>(p, F, cur, cnt, (int)(rd & 1u), nxt, lc + (rd + 1) % 3, g0, rows, cta, sh_q[wid],
                                 sh_e[wid]);
-      if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
+      if ((quit = team_sync<ONE>(ctl, p.ctas, gen, p.err))) break;
       const uint32_t nc = __ldcg(lc + (rd + 1) % 3);
       if (nc == 0u) break;  // uniform: not written before the next barrier
-      pop_redraw<WGT>(p, F, K, nxt, nc, cur, cnt, (int)((rd + 1) & 1u), g0, cta);
+      pop_redraw<WGT, BAT>(p, F, K, nxt, nc, cur, cnt, (int)((rd + 1) & 1u), g0, cta);
       cnt = nc;
-      if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;
+      if ((quit = team_sync<ONE>(ctl, p.ctas, gen, p.err))) break;
     }
     if (quit) break;
     if (p.parents != nullptr) {
@@ -544,9 +556,9 @@ __global__ void __launch_bounds__(PK_T, 4) k_pop(PopParams p) {
         const int64_t r = i / p.n;
         p.parents[g0 * p.n + i] = (int32_t)(F[r * p.ld + (i - r * p.n)] & PW_ID);
       }
-      if (p.item_ns != nullptr) pop_stamp(p, g0, rows, cta);  // the parents are part of the trees
+      if (BAT) pop_stamp(p, g0, rows, cta);  // the parents are part of the trees
     }
-    if ((quit = team_sync(ctl, p.ctas, gen, p.err))) break;  // the tops are read before they are drawn again
+    if ((quit = team_sync<ONE>(ctl, p.ctas, gen, p.err))) break;  // the tops are read before they are drawn again
   }
   pop_stats(p, pops);
 }
@@ -583,8 +595,11 @@ constexpr int64_t POP_WINDOW = 640ll << 20;  // bytes of tops, all teams
 // 6.8 / 6.8; BA 2^20, 1024 trees 21.7 / 20.4 / 28.8 / 45.3.
 constexpr int32_t POP_MANY_N = 1 << 17;  // every CTA a team up to this size, and for rooted graphs
 
+template <bool ONE>
 static const void* pop_fn(const fc_graph* g) {
-  return g->weighted ? (const void*)k_pop<true> : (const void*)k_pop<false>;
+  if (g->num_graphs > 0)
+    return g->weighted ? (const void*)k_pop<true, true, ONE> : (const void*)k_pop<false, true, ONE>;
+  return g->weighted ? (const void*)k_pop<true, false, ONE> : (const void*)k_pop<false, false, ONE>;
 }
 
 fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* pl) {
@@ -592,7 +607,7 @@ fc_status pop_plan(const fc_graph* g, int64_t total, PopPlan* pl) {
   FC_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device));
   FC_CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device));
   if (per_sm == 0) {  // of the kernel and the device alone
-    FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pop_fn(g), PK_T, 0));
+    FC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pop_fn<false>(g), PK_T, 0));
     g->pop_per_sm.store(per_sm, std::memory_order_relaxed);
   }
   if (!coop || per_sm < 1) {
@@ -662,8 +677,8 @@ fc_status pop_sample(fc_graph* g, const WParams& w, const PopPlan& pl, void* ws,
   void* args[] = {&p};
   const dim3 grid((unsigned)(pl.teams * pl.ctas));
   // teams of one CTA wait for no other: no cooperative launch
-  FC_CK(pl.ctas == 1 ? cudaLaunchKernel(pop_fn(g), grid, dim3(PK_T), args, 0, st)
-                     : cudaLaunchCooperativeKernel(pop_fn(g), grid, dim3(PK_T), args, 0, st));
+  FC_CK(pl.ctas == 1 ? cudaLaunchKernel(pop_fn<true>(g), grid, dim3(PK_T), args, 0, st)
+                     : cudaLaunchCooperativeKernel(pop_fn<false>(g), grid, dim3(PK_T), args, 0, st));
   FC_LAUNCHED();
   g->last_W = PK_T;
   g->last_regs = 64;

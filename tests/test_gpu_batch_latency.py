@@ -1,6 +1,6 @@
 """Per-graph completion times of a batch (fc_batch_latency) under the
 cycle-popping sampler: a graph is complete when the last cycle of its last
-tree is redrawn, not when the launch ends."""
+tree is found, not when the launch ends."""
 import numpy as np
 import pytest
 
