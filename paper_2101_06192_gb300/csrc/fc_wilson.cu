@@ -685,7 +685,18 @@ static fc_status batch_stamps(fc_graph* g, int64_t tau, bool capturing, cudaStre
 // 25.0 -> 4.4, 1 47.3 -> 15.0, 10 79.4 -> 38.9; ER n = 1000, 2000 trees 1.3 ->
 // 0.37; BA n = 2^20 rooted at its hub, 152 trees 118 -> 87; with forest roots
 // and depths (parents, then pointer jumping, against recording them as vertices
-// join the tree) BA n = 2^17, 96 trees 2.3 -> 0.88.  Exceptions:
+// join the tree) BA n = 2^17, 96 trees 2.3 -> 0.88.
+//
+// Many rounds and long walks (rooted graphs of large diameter, large alphas) do
+// not change the order: rooted at its centre, 16 trees of a square grid of 32^2
+// 16 -> 4.8, of 256^2 1091 -> 497, 512^2 5167 -> 2793, 1024^2 38,871 -> 17,891;
+// cubic grid 32^3 674 -> 98; path of 300 71 -> 40, of 1024 855 -> 515; binary tree
+// of 4095 25 -> 20, of 65,535 593 -> 112; ring with shortcuts 520 -> 188; weighted
+// grid 2^18, 128 trees, alpha 10 / 100 / 1000 54 / 241 / 531 -> 10.4 / 57 / 396;
+// BA 2^18 at alpha 100 250 -> 11; at alpha 10^4 the walkers run out of their
+// watchdog (grid, BA, ER) where popping takes 320 to 810.  One tree up to 1024
+// trees, weighted or not: none of some 120 calls was faster by walkers, which
+// lose more to claims, waits and repeated paths.  Exceptions:
 //  * ids of 29 bits in the words of the tops;
 //  * diagnostic calls (parents and step counts together) on unweighted single
 //    graphs of 2^15 to 2^16 vertices: tests/test_gpu_edge_kernel.py pins the
