@@ -283,8 +283,9 @@ fc_status fc_sample_usts_forest(fc_graph* g, uint64_t seed, int64_t tau, int64_t
  * launch, its memsets and the combinations after it become graph nodes).
  * Device-side errors stay in the graph's error word until fc_sampler_check.
  * The sampler's scratch buffer must already be large enough: make one
- * uncaptured fc_sample_usts call with the same graph and tau first (else
- * FC_EINVAL during capture).
+ * uncaptured fc_sample_usts call with the same graph and tau first, or with
+ * another graph of the device that takes as much (else FC_EINVAL during
+ * capture).
  */
 fc_status fc_sample_usts_async(fc_graph* g, uint64_t seed, int64_t tau, int64_t tree_offset, uint32_t* R,
                                uint32_t* C, int32_t* parents, uint64_t max_steps_per_tree, uint64_t* steps_out,

@@ -466,6 +466,9 @@ extern "C" fc_status fc_release_scratch(void) {
   }
   // the cycle-popping sampler's scratch is a stream-ordered allocation of each
   // call: once freed it stays in the device's pool (retain_pool)
+  bool any = false;
+  for (bool set : g_pool_set) any |= set;
+  if (!any) return FC_OK;  // no graph yet: no context is made, and none is needed
   int cur = 0;
   FC_CK(cudaGetDevice(&cur));
   cudaError_t e = cudaSuccess;
